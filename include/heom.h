@@ -97,9 +97,9 @@ extern "C" {
                                 auxiliaries of different depths become of comparable size (the
                                 first step towards filtering small ones, which this library does
                                 not do).  heom_get_state/heom_set_state exchange sigma~_n.  For
-                                N <= 8 not with the register node view (node_threads 1 or 2) nor
-                                with mode 2: the default launch shape avoids them, and a launch
-                                shape set to them fails at propagate time with HEOM_EUNSUPPORTED */
+                                N <= 8 not with node_threads 1 or 2 nor with mode 2: the
+                                default launch shape avoids them, and a launch shape set to
+                                them fails at propagate time with HEOM_EUNSUPPORTED */
 
 /* largest supported number of sites and of hierarchy nodes per instance */
 #define HEOM_MAX_SITES 24
@@ -281,17 +281,20 @@ int heom_ctx_num_nodes(const heom_ctx* ctx, int64_t* out);
  * mode 3 team_ctas is the number of nodes each thread carries, 1..6 (more
  * than one: real H and 4..8 sites only, HEOM_EUNSUPPORTED otherwise), which
  * lets a hierarchy of up to about 6800 nodes (N = 7) run with all CTAs
- * resident.  Mode 3 is the default for one hierarchy of 256 nodes or more
- * when all its CTAs fit on the GPU at once with some number of nodes per
- * thread (the fewest that fit).  block_threads: multiple of 32, 64..512
+ * resident; with more than three (two at N = 8) the throughput engine of mode 1
+ * runs in its place, which is faster there.  Mode 3 is the default for one
+ * hierarchy of 256 nodes or more when all its CTAs fit on the GPU at once with
+ * some number of nodes per thread (the fewest that fit).  block_threads: multiple of 32, 64..512
  * (64..256 for HEOM_FP64, whose kernels are compiled for that register budget);
  * in mode 3 the CTA size, at most 384 with one node per thread and 256 with
  * more, of which every N(N+1)/2 threads make a row of team_ctas nodes (N = 7,
  * one node per thread: 12 nodes in 336 threads); a call whose CTAs cannot all
  * be resident fails with HEOM_EINVAL.  Switching between mode 3 and the
  * other modes without giving team_ctas or block_threads resets them to that
- * family's default.  node_threads: threads sharing one node's matrix, 1..32
- * (1 or 2 keep the node's matrix in registers; not used by mode 3).  A
+ * family's default.  node_threads: threads sharing one node's matrix, 1..32;
+ * 1, 2 and 4 select, in modes 0 and 1 with N <= 8, the throughput engine, which
+ * gives a node N threads and a CTA about twice block_threads threads whatever
+ * the count (scaled hierarchies: 4 only); not used by mode 3.  A
  * negative mode or a non-positive value keeps the current setting. */
 int heom_set_launch(heom_ctx* ctx, int32_t mode, int32_t team_ctas, int32_t block_threads, int32_t node_threads);
 int heom_get_launch(const heom_ctx* ctx, int32_t* mode, int32_t* team_ctas, int32_t* block_threads,

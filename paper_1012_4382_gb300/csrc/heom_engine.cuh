@@ -11,12 +11,12 @@
 // Storage.  Every sigma_n is Hermitian (the right-hand side maps Hermitian
 // matrices to Hermitian ones), so a node is stored as N*N reals: element
 // (a, b) of the packed matrix P holds Re sigma_ab for a <= b and Im sigma_ba
-// for a > b.  Arrays are element-major ("structure of arrays"):
-// w[p * Mpad + n] is packed element p of node n, so a warp that handles 32
+// for a > b.  Arrays are in blocks of 32 nodes, each element of a block
+// contiguous over its nodes (see node_col), so a warp that handles 32
 // consecutive nodes reads and writes every element with one 128-byte
-// (float) or 256-byte (double) transaction, and neighbour gathers
-// w[p * Mpad + up_j(n)] touch ascending, nearly contiguous addresses because
-// n -> n + e_j preserves the lexicographic order inside a level.
+// (float) or 256-byte (double) transaction, and neighbour gathers from a warp
+// touch ascending, nearly contiguous addresses because n -> n + e_j preserves
+// the lexicographic order inside a level.
 //
 // Time stepping.  The right-hand side is linear and autonomous, so classic
 // RK4 (App. B) is the degree-4 Taylor polynomial of h L.  It is evaluated in
@@ -30,20 +30,15 @@
 // same holds for the radiative loss with Gamma_phot.
 //
 // Parallel decomposition.  A "team" (one thread-block cluster, or the whole
-// grid) owns one hierarchy at a time.  Nodes are grouped in blocks of 32
-// (one warp lane per node); each node block is split into G "unit groups"
-// (1 <= G <= 32): warp (block, g) computes the packed elements whose unit
-// index u satisfies u % G == g.  Units are the N(N-1)/2 off-diagonal pairs
-// (two packed reals each) and the N diagonal entries.  With G <= 2 a thread
-// loads its node's whole packed matrix into registers once (RegView); with
-// larger G each unit loads the elements it needs (LoadView), so many short
-// threads share a node.  All index arithmetic on the packed matrix is resolved
-// at compile time.  Between RK4 stages the team synchronises with a hardware
-// cluster barrier (release/acquire at cluster scope) or a software grid
-// barrier with a bounded wait.  In mixed precision the root node rho is
-// split into one work item per unit, each run by one lane of its own warp,
-// so that its double-precision accumulations (FP64 runs at 1/64 of the FP32
-// rate on this GPU) proceed in parallel rather than in one serial chain.
+// grid) owns one hierarchy at a time.  This file's kernels are the load views:
+// nodes are grouped in blocks of 32 (one warp lane per node), and each node
+// block is split into G "unit groups" (1 <= G <= 32): warp (block, g) computes
+// the packed elements whose unit index u satisfies u % G == g.  Units are the
+// N(N-1)/2 off-diagonal pairs (two packed reals each) and the N diagonal
+// entries; each loads the elements it needs.  They serve the group counts the
+// throughput engine (heom_block.cuh) does not take.  Between RK4 stages the team
+// synchronises with a hardware cluster barrier (release/acquire at cluster
+// scope) or a software grid barrier with a bounded wait.
 #pragma once
 
 #include <cstdint>
@@ -65,10 +60,10 @@ struct Inst {
   int32_t N, K, M, Mpad;
   int32_t complex_h, terminator;
   int32_t wstride;     // scaled hierarchy: K + 2, the row length of wsc
-  int32_t pad1;
+  int32_t rstride;     // stride between the root's elements in a state array: 32 (N <= 8), Mpad (N > 8)
   const int32_t* up;   // [N][Mpad] index of n + e_j or -1
   const int32_t* dn;   // [N][Mpad] (n_j << 24) | index of n - e_j, or -1
-  void* y;             // [N*N][Mpad] packed state, element-major (R)
+  void* y;             // packed state (R), see state_elem; N <= 8: ended by a block of zeros
   void* wa;            // stage buffers, same layout
   void* wb;
   // mixed precision: the root node rho in float-float, N*N (hi, lo) float
@@ -147,6 +142,22 @@ __device__ __forceinline__ void static_for(F&& f) {
     f(std::integral_constant<int, B>{});
     static_for<B + 1, E>(f);
   }
+}
+
+// Layout of a state array.  N <= 8: blocks of 32 nodes, [Mpad/32][N*N][32] --
+// element p of node n at node_col<N>(n) + 32 p, so that every element of a
+// node (and of a neighbour) is at a compile-time offset from one address --
+// followed by one more block that stays zero, which absent neighbours read.
+// N > 8: element-major, [N*N][Mpad].
+template <int N>
+__host__ __device__ __forceinline__ constexpr unsigned node_col(int n) {
+  return (unsigned)(n >> 5) * (N * N * 32) + (n & 31);
+}
+__host__ __device__ __forceinline__ size_t state_elem(int N, int Mpad, int p, int64_t n) {
+  return N <= kMaxSmallN ? ((size_t)(n >> 5) * (N * N) + p) * 32 + (n & 31) : (size_t)p * Mpad + n;
+}
+__host__ __device__ __forceinline__ size_t state_reals(int N, int Mpad) {
+  return (size_t)N * N * (N <= kMaxSmallN ? Mpad + 32 : Mpad);
 }
 
 // pair index u -> (a, b), a < b, in the order (0,1),(0,2),...,(1,2),...
@@ -231,11 +242,11 @@ __device__ __forceinline__ bool team_barrier(const EngineArgs& A, unsigned& epoc
 //   Nj<j>()       n_j
 //   G<p>(h)       packed element p of the linked node h's stage input
 //   Y<p>(), St<p>(v)  the node's y element, and the store of its stage output
-// Global views address the element-major arrays in device memory; shared
-// views address one thread-block cluster's distributed shared memory, where
-// each CTA holds a contiguous slice of the nodes and link handles are
-// shared::cluster addresses.  "Reg" views load the node's whole packed matrix
-// into registers once; "Load" views load each element where a unit uses it.
+// Global views address the state arrays in device memory; shared views address
+// one thread-block cluster's distributed shared memory, where each CTA holds a
+// contiguous slice of the nodes and link handles are shared::cluster
+// addresses.  Each element is loaded where a unit uses it (the shared view may
+// load the node's whole packed matrix into registers once).
 
 // Loads *a when q holds, else returns 0; predicated, so that gathers of
 // absent neighbours need no branch.
@@ -263,65 +274,34 @@ struct GlobalArrays {
   int Mp;
 };
 
-template <int N, typename R, bool REG>
+template <int N, typename R>
 struct GlobalView {
-  const R* __restrict__ win;  // column n of the input
+  const R* __restrict__ win;  // column of node n of the input
   const R* __restrict__ base;  // input, for gathers
   R* __restrict__ wout;
   const R* __restrict__ y;
   const int32_t* __restrict__ upt;
   const int32_t* __restrict__ dnt;
   int Mp;
-  R sg[REG ? N * N : 1];
-  int upr[REG ? N : 1], dnr[REG ? N : 1];
   __device__ __forceinline__ GlobalView(const GlobalArrays<R>& a, int n)
-      : win(a.win + n), base(a.win), wout(a.wout + n), y(a.y + n), upt(a.up + n), dnt(a.dn + n), Mp(a.Mp) {
-    if constexpr (REG) {
-#pragma unroll
-      for (int p = 0; p < N * N; ++p) sg[p] = win[p * Mp];
-#pragma unroll
-      for (int j = 0; j < N; ++j) {
-        upr[j] = upt[j * Mp];
-        dnr[j] = dnt[j * Mp];
-      }
-    }
-  }
+      : win(a.win + node_col<N>(n)), base(a.win), wout(a.wout + node_col<N>(n)), y(a.y + node_col<N>(n)), upt(a.up + n),
+        dnt(a.dn + n), Mp(a.Mp) {}
   template <int p>
-  __device__ __forceinline__ R P() const {
-    if constexpr (REG) return sg[p];
-    else return win[p * Mp];
-  }
+  __device__ __forceinline__ R P() const { return win[p * 32]; }
   template <int j>
-  __device__ __forceinline__ int Up() const {
-    if constexpr (REG) return upr[j];
-    else return upt[j * Mp];
-  }
+  __device__ __forceinline__ int Up() const { return upt[j * Mp]; }
   template <int j>
-  __device__ __forceinline__ int DnRaw() const {
-    if constexpr (REG) return dnr[j];
-    else return dnt[j * Mp];
-  }
+  __device__ __forceinline__ int Dn() const { return Dnr(j); }
   template <int j>
-  __device__ __forceinline__ int Dn() const {
-    const int d = DnRaw<j>();
-    return d < 0 ? -1 : (d & 0xFFFFFF);
-  }
-  template <int j>
-  __device__ __forceinline__ R Nj() const {
-    const int d = DnRaw<j>();
-    return d < 0 ? R(0) : R(d >> 24);
-  }
+  __device__ __forceinline__ R Nj() const { return Njr(j); }
   template <int p>
-  __device__ __forceinline__ R G(int h) const { return base[p * Mp + h]; }
-  // element p of node h, or 0 when h == -1 (no link)
+  __device__ __forceinline__ R G(int h) const { return base[node_col<N>(h) + p * 32]; }
   template <int p>
-  __device__ __forceinline__ R G0(int h) const { return ld_global_or0(base + (p * Mp + h), h != -1); }
+  __device__ __forceinline__ R Y() const { return y[p * 32]; }
   template <int p>
-  __device__ __forceinline__ R Y() const { return y[p * Mp]; }
-  template <int p>
-  __device__ __forceinline__ void St(R v) const { wout[p * Mp] = v; }
-  // the same with run-time indices (load views)
-  __device__ __forceinline__ R Pr(int p) const { return win[p * Mp]; }
+  __device__ __forceinline__ void St(R v) const { wout[p * 32] = v; }
+  // the same with run-time indices
+  __device__ __forceinline__ R Pr(int p) const { return win[p * 32]; }
   __device__ __forceinline__ int Upr(int j) const { return upt[j * Mp]; }
   __device__ __forceinline__ int Dnr(int j) const {
     const int d = dnt[j * Mp];
@@ -331,19 +311,10 @@ struct GlobalView {
     const int d = dnt[j * Mp];
     return d < 0 ? R(0) : R(d >> 24);
   }
-  __device__ __forceinline__ R Gr(int p, int h) const { return base[p * Mp + h]; }
-  __device__ __forceinline__ R Yr(int p) const { return y[p * Mp]; }
-  __device__ __forceinline__ void Str(int p, R v) const { wout[p * Mp] = v; }
+  __device__ __forceinline__ R Gr(int p, int h) const { return base[node_col<N>(h) + p * 32]; }
+  __device__ __forceinline__ R Yr(int p) const { return y[p * 32]; }
+  __device__ __forceinline__ void Str(int p, R v) const { wout[p * 32] = v; }
 };
-
-__device__ __forceinline__ float ld_dsmem_f32_or0(unsigned addr, bool q) {
-  float v = 0.f;
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q ld.shared::cluster.f32 %0, [%1];\n\t}"
-               : "+f"(v)
-               : "r"(addr), "r"((unsigned)q)
-               : "memory");
-  return v;
-}
 
 __device__ __forceinline__ float ld_dsmem_f32(unsigned addr) {
   float v;
@@ -410,10 +381,6 @@ struct SmemView {
   template <int p>
   __device__ __forceinline__ float G(int h) const {
     return ld_dsmem_f32((unsigned)h + win_off + (unsigned)(p * B * 4));
-  }
-  template <int p>
-  __device__ __forceinline__ float G0(int h) const {
-    return ld_dsmem_f32_or0((unsigned)h + win_off + (unsigned)(p * B * 4), h != -1);
   }
   template <int p>
   __device__ __forceinline__ float Y() const { return y[p * B]; }
@@ -654,20 +621,13 @@ __device__ __forceinline__ R scaled_dn(const R* __restrict__ w, int S, int j, R 
 // Right-hand side of unit u (pair (a, b) or diagonal a) of one node.
 // Returns the real part in re and, for pairs, the imaginary part in im.
 // J is symmetric and Ji antisymmetric, so all the coefficients of a unit sit
-// in rows a and b and in the site records of a and b.  tc[j] is the
-// terminator factor (n_j + 1) / (ngam + gamma_j) of a leaf node (term), 0
-// elsewhere.  BF: branch-free form -- absent neighbours read as 0 (predicated
-// loads), n_j is 0 where there is no down link and the terminator terms are
-// always evaluated, so the compiler may issue the loads of several units
-// ahead of their arithmetic; worth it where a thread runs many units of a
-// node and arithmetic is cheap (FP32, unit groups G <= 2).  Otherwise each
-// term is skipped where it is absent, which saves FP64 instructions (1/64
-// rate) and the latency of unneeded loads when a thread runs one unit.
-// SC: scaled hierarchy, link weights from wsc (row length ws); branching form only.
-template <int N, int u, typename R, bool CPLX, bool BF, bool SC, class V>
-__device__ __forceinline__ void unit_rhs(const V& v, const R* __restrict__ cf, R ngam, bool term, const R* tc, R& re,
-                                         R& im, const R* __restrict__ wsc, int ws) {
-  static_assert(!(SC && BF), "the scaled hierarchy uses the branching form");
+// in rows a and b and in the site records of a and b.  term: the Markov
+// terminator of a leaf node.  Each term is skipped where it is absent, which
+// saves FP64 instructions (1/64 rate) and the latency of unneeded loads.
+// SC: scaled hierarchy, link weights from wsc (row length ws).
+template <int N, int u, typename R, bool CPLX, bool SC, class V>
+__device__ __forceinline__ void unit_rhs(const V& v, const R* __restrict__ cf, R ngam, bool term, R& re, R& im,
+                                         const R* __restrict__ wsc, int ws) {
   using L = CoefLayout<R>;
   constexpr int NP = N * (N - 1) / 2;
   constexpr int JS = L::JS(N);
@@ -731,62 +691,45 @@ __device__ __forceinline__ void unit_rhs(const V& v, const R* __restrict__ cf, R
     // down-couplings n_j theta_j sigma_{n-e_j}
     const int da = v.template Dn<a>();
     const int db = v.template Dn<b>();
-    if constexpr (BF) {
-      const R uar = v.template G0<pab>(ua), uai = v.template G0<pba>(ua);
-      const R ubr = v.template G0<pab>(ub), ubi = v.template G0<pba>(ub);
-      const R dar = v.template G0<pab>(da), dai = v.template G0<pba>(da);
-      const R dbr = v.template G0<pab>(db), dbi = v.template G0<pba>(db);
-      re += ubi - uai;
-      im += uar - ubr;
-      // terminator: sigma_{n+e_j} ~ (n_j+1)/(ngam+gamma_j) theta_j sigma_n, then i V_j^x of it
-      const R ca = tc[a], cb = tc[b];
+    if (ua != -1) {
+      R gr = v.template G<pba>(ua), gi = v.template G<pab>(ua);
+      if constexpr (SC) {
+        const R w = scaled_up(wsc, ws, a, v.template Nj<a>());
+        gr *= w;
+        gi *= w;
+      }
+      re -= gr;
+      im += gi;
+    }
+    if (ub != -1) {
+      R gr = v.template G<pba>(ub), gi = v.template G<pab>(ub);
+      if constexpr (SC) {
+        const R w = scaled_up(wsc, ws, b, v.template Nj<b>());
+        gr *= w;
+        gi *= w;
+      }
+      re += gr;
+      im -= gi;
+    }
+    if (term) {
+      const R ca = (v.template Nj<a>() + R(1)) / (ngam + cf[L::gam(N) + a]);
+      const R cb = (v.template Nj<b>() + R(1)) / (ngam + cf[L::gam(N) + b]);
       re += ca * (-al_a * x - be_a * yi) + cb * (-al_b * x + be_b * yi);
       im += ca * (-al_a * yi + be_a * x) + cb * (-al_b * yi - be_b * x);
-      const R n_a = v.template Nj<a>();
-      const R n_b = v.template Nj<b>();
-      re += n_a * (be_a * dar - al_a * dai) + n_b * (be_b * dbr + al_b * dbi);
-      im += n_a * (al_a * dar + be_a * dai) + n_b * (be_b * dbi - al_b * dbr);
-    } else {
-      if (ua != -1) {
-        R gr = v.template G<pba>(ua), gi = v.template G<pab>(ua);
-        if constexpr (SC) {
-          const R w = scaled_up(wsc, ws, a, v.template Nj<a>());
-          gr *= w;
-          gi *= w;
-        }
-        re -= gr;
-        im += gi;
-      }
-      if (ub != -1) {
-        R gr = v.template G<pba>(ub), gi = v.template G<pab>(ub);
-        if constexpr (SC) {
-          const R w = scaled_up(wsc, ws, b, v.template Nj<b>());
-          gr *= w;
-          gi *= w;
-        }
-        re += gr;
-        im -= gi;
-      }
-      if (term) {
-        const R ca = (v.template Nj<a>() + R(1)) / (ngam + cf[L::gam(N) + a]);
-        const R cb = (v.template Nj<b>() + R(1)) / (ngam + cf[L::gam(N) + b]);
-        re += ca * (-al_a * x - be_a * yi) + cb * (-al_b * x + be_b * yi);
-        im += ca * (-al_a * yi + be_a * x) + cb * (-al_b * yi - be_b * x);
-      }
-      if (da != -1) {
-        const R n_a = SC ? scaled_dn(wsc, ws, a, v.template Nj<a>()) : v.template Nj<a>();
-        const R yr = v.template G<pab>(da);
-        const R yy = v.template G<pba>(da);
-        re += n_a * (be_a * yr - al_a * yy);
-        im += n_a * (al_a * yr + be_a * yy);
-      }
-      if (db != -1) {
-        const R n_b = SC ? scaled_dn(wsc, ws, b, v.template Nj<b>()) : v.template Nj<b>();
-        const R yr = v.template G<pab>(db);
-        const R yy = v.template G<pba>(db);
-        re += n_b * (be_b * yr + al_b * yy);
-        im += n_b * (be_b * yy - al_b * yr);
-      }
+    }
+    if (da != -1) {
+      const R n_a = SC ? scaled_dn(wsc, ws, a, v.template Nj<a>()) : v.template Nj<a>();
+      const R yr = v.template G<pab>(da);
+      const R yy = v.template G<pba>(da);
+      re += n_a * (be_a * yr - al_a * yy);
+      im += n_a * (al_a * yr + be_a * yy);
+    }
+    if (db != -1) {
+      const R n_b = SC ? scaled_dn(wsc, ws, b, v.template Nj<b>()) : v.template Nj<b>();
+      const R yr = v.template G<pab>(db);
+      const R yy = v.template G<pba>(db);
+      re += n_b * (be_b * yr + al_b * yy);
+      im += n_b * (be_b * yy - al_b * yr);
     }
   } else {
     constexpr int a = u - NP;
@@ -811,13 +754,9 @@ __device__ __forceinline__ void unit_rhs(const V& v, const R* __restrict__ cf, R
     }
     re -= (ngam + R(2) * cf[L::gd(N) + a]) * x;
     const int da = v.template Dn<a>();
-    if constexpr (BF) {
-      re += R(2) * v.template Nj<a>() * sa[3] * v.template G0<paa>(da);
-    } else {
-      if (da != -1) {
-        const R n_a = SC ? scaled_dn(wsc, ws, a, v.template Nj<a>()) : v.template Nj<a>();
-        re += R(2) * n_a * sa[3] * v.template G<paa>(da);
-      }
+    if (da != -1) {
+      const R n_a = SC ? scaled_dn(wsc, ws, a, v.template Nj<a>()) : v.template Nj<a>();
+      re += R(2) * n_a * sa[3] * v.template G<paa>(da);
     }
   }
 }
@@ -829,167 +768,72 @@ struct OutStep {
   int64_t row;
 };
 
-// Does unit u belong to this item's group?  GS > 0: the group is u % GS ==
-// GI, known at compile time; GS == 0: the runtime mask umask decides.
-template <int GS, int GI, int u>
-__host__ __device__ constexpr bool in_group(uint64_t umask) {
-  if constexpr (GS > 0) return (u % GS) == GI;
-  else return (umask >> u) & 1ull;
-}
-
-// Shared-memory scratch of one warp for the staged outputs of the global
-// engine: element p of lane l at stg[p * 32 + l]; per CTA the root's
-// float-float stage outputs and its population row.
-template <typename R>
-struct Staging {
-  R* stg;        // this lane's column
-  FF* root_ff;   // [N*N]
-  double* pops;  // [N]
-};
-
-// All units of one node in this item's group, one RK4 stage.  For the root
-// node of the mixed path the Horner update w = y + h r runs in float-float
-// on the root's own buffers, and the hi part is stored for the neighbours.
-// At the last stage the owner of the root's diagonal unit a adds
-// h Gamma_a x_aa to its running eta and loss sums (the extra rows of the
-// augmented RK4 system, x being the stage input).  ROOT: the node may be the
-// root (only the item holding node 0 needs that code).  With staging the
-// results first go to shared memory and are copied out after the last unit,
-// so no global store separates the loads of one unit from those of the next
-// (STG; without it the results are stored where they are computed).
-template <int N, typename R, bool MIXED, bool CPLX, int GS, int GI, bool ROOT, bool STG, bool BF, bool SC, class V>
+// All units of one node in umask, one RK4 stage.  For the root node of the
+// mixed path the Horner update w = y + h r runs in float-float on the root's
+// own buffers, and the hi part is stored for the neighbours.  At the last
+// stage the owner of the root's diagonal unit a adds h Gamma_a x_aa to its
+// running eta and loss sums (the extra rows of the augmented RK4 system, x
+// being the stage input).
+template <int N, typename R, bool MIXED, bool CPLX, bool SC, class V>
 __device__ __forceinline__ void node_units(const Inst& I, const R* __restrict__ cf, const double* __restrict__ cfd,
                                            const StageCoef<R>& P, const V& v, R ngam, int s, bool root,
-                                           uint64_t umask, OutStep os, EtaAcc<R>& ea, const Staging<R>& sg) {
-  using L = CoefLayout<R>;
+                                           uint64_t umask, OutStep os, EtaAcc<R>& ea) {
   constexpr int NP = N * (N - 1) / 2;
   constexpr int U = NP + N;
-  constexpr bool stage_out = STG;
-  // terminator factors: precomputed for the branch-free form, else computed where used
-  R tc[BF ? N : 1];
-#pragma unroll
-  for (int j = 0; j < (BF ? N : 1); ++j) tc[j] = R(0);
   const bool term = I.terminator && v.template Up<0>() == -1;
-  if constexpr (BF) {
-    if (term) {
-      static_for<0, N>([&](auto jc) {
-        constexpr int j = decltype(jc)::value;
-        tc[j] = (v.template Nj<j>() + R(1)) / (ngam + cf[L::gam(N) + j]);
-      });
-    }
-  }
-  const bool out_row = ROOT && (s == 3) && root && I.out_pops && os.now;
-  auto put = [&](auto pc, R w) {
-    constexpr int p = decltype(pc)::value;
-    if constexpr (stage_out) sg.stg[p * 32] = w;
-    else v.template St<p>(w);
-  };
+  const bool out_row = (s == 3) && root && I.out_pops && os.now;
 
   static_for<0, U>([&](auto uc) {
     constexpr int u = decltype(uc)::value;
-    if constexpr (GS > 0) {
-      if constexpr (!in_group<GS, GI, u>(0)) return;
-    } else {
-      if (!in_group<0, 0, u>(umask)) return;
-    }
+    if (!((umask >> u) & 1ull)) return;
     R re, im;
-    unit_rhs<N, u, R, CPLX, BF, SC>(v, cf, ngam, term, tc, re, im, static_cast<const R*>(I.wsc), I.wstride);
+    unit_rhs<N, u, R, CPLX, SC>(v, cf, ngam, term, re, im, static_cast<const R*>(I.wsc), I.wstride);
     if constexpr (u < NP) {
       constexpr int a = pair_a(N, u);
       constexpr int b = pair_b(N, u);
       constexpr int pr = a * N + b, pi = b * N + a;
       R wr, wi;
-      if constexpr (ROOT && MIXED) {
-        if (root) {
+      if (MIXED && root) {
+        if constexpr (MIXED) {
           const FF fr = ff_axpy(P.root_y[pr], P.h, P.hl, re);
           const FF fi = ff_axpy(P.root_y[pi], P.h, P.hl, im);
-          if constexpr (stage_out) {
-            sg.root_ff[pr] = fr;
-            sg.root_ff[pi] = fi;
-          } else {
-            P.root_out[pr] = fr;
-            P.root_out[pi] = fi;
-          }
+          P.root_out[pr] = fr;
+          P.root_out[pi] = fi;
           wr = fr.h;
           wi = fi.h;
-        } else {
-          wr = v.template Y<pr>() + P.h * re;
-          wi = v.template Y<pi>() + P.h * im;
         }
       } else {
         wr = v.template Y<pr>() + P.h * re;
         wi = v.template Y<pi>() + P.h * im;
       }
-      put(std::integral_constant<int, pr>{}, wr);
-      put(std::integral_constant<int, pi>{}, wi);
+      v.template St<pr>(wr);
+      v.template St<pi>(wi);
     } else {
       constexpr int a = u - NP;
       constexpr int pd = a * N + a;
       R w;
-      [[maybe_unused]] double pop = 0.0;
-      if constexpr (ROOT && MIXED) {
-        if (root) {
+      double pop = 0.0;
+      if (MIXED && root) {
+        if constexpr (MIXED) {
           if (s == 3) ea.add(I, a, P.root_in[pd]);
           if (s == 2) ea.add_xi(I, a, P.root_in[pd]);
           const FF f = ff_axpy(P.root_y[pd], P.h, P.hl, re);
-          if constexpr (stage_out) sg.root_ff[pd] = f;
-          else P.root_out[pd] = f;
+          P.root_out[pd] = f;
           w = f.h;
           if (out_row) pop = ff_to_double(f);
-        } else {
-          w = v.template Y<pd>() + P.h * re;
         }
       } else {
-        if constexpr (ROOT && !MIXED) {
+        if constexpr (!MIXED) {
           if (root && s == 3) ea.add(I, cfd, N, a, (double)v.template P<pd>());
           if (root && s == 2) ea.add_xi(I, cfd, a, (double)v.template P<pd>());
         }
         w = v.template Y<pd>() + P.h * re;
-        if constexpr (ROOT) {
-          if (out_row) pop = (double)w;
-        }
+        if (out_row) pop = (double)w;
       }
-      put(std::integral_constant<int, pd>{}, w);
-      if constexpr (ROOT) {
-        if (out_row) {
-          if constexpr (stage_out) sg.pops[a] = pop;
-          else I.out_pops[os.row * N + a] = pop;
-        }
-      }
+      v.template St<pd>(w);
+      if (out_row) I.out_pops[os.row * N + a] = pop;
     }
   });
-
-  if constexpr (stage_out) {
-    static_for<0, U>([&](auto uc) {
-      constexpr int u = decltype(uc)::value;
-      if constexpr (GS > 0) {
-        if constexpr (!in_group<GS, GI, u>(0)) return;
-      } else {
-        if (!in_group<0, 0, u>(umask)) return;
-      }
-      if constexpr (u < NP) {
-        constexpr int pr = pair_a(N, u) * N + pair_b(N, u), pi = pair_b(N, u) * N + pair_a(N, u);
-        v.template St<pr>(sg.stg[pr * 32]);
-        v.template St<pi>(sg.stg[pi * 32]);
-        if constexpr (ROOT && MIXED) {
-          if (root) {
-            P.root_out[pr] = sg.root_ff[pr];
-            P.root_out[pi] = sg.root_ff[pi];
-          }
-        }
-      } else {
-        constexpr int a = u - NP;
-        constexpr int pd = a * N + a;
-        v.template St<pd>(sg.stg[pd * 32]);
-        if constexpr (ROOT) {
-          if constexpr (MIXED) {
-            if (root) P.root_out[pd] = sg.root_ff[pd];
-          }
-          if (out_row) I.out_pops[os.row * N + a] = sg.pops[a];
-        }
-      }
-    });
-  }
 }
 
 // ------------------------------------------------ run-time indexed units
@@ -999,7 +843,7 @@ __device__ __forceinline__ void node_units(const Inst& I, const R* __restrict__ 
 // unrolled unit bodies would then put the code of all N(N+1)/2 units in the
 // instruction stream of one SM (tens of KB, more than the instruction cache
 // holds); these versions run one compact body with the unit's (a, b) known at
-// run time.  Same arithmetic as unit_rhs (branching form).
+// run time.  Same arithmetic as unit_rhs.
 __device__ __forceinline__ void unit_pair_of(int N, int u, int& a, int& b) {
   a = 0;
   while (u >= N - 1 - a) {
@@ -1163,18 +1007,17 @@ struct CachedView {
   const R* __restrict__ base;
   R* __restrict__ wout;
   const R* __restrict__ y;
-  int Mp;
   const CachedUnit<R>& c;
   __device__ __forceinline__ CachedView(const GlobalArrays<R>& g, const CachedUnit<R>& cu)
-      : win(g.win + cu.n), base(g.win), wout(g.wout + cu.n), y(g.y + cu.n), Mp(g.Mp), c(cu) {}
-  __device__ __forceinline__ R Pr(int p) const { return win[p * Mp]; }
+      : win(g.win + node_col<N>(cu.n)), base(g.win), wout(g.wout + node_col<N>(cu.n)), y(g.y + node_col<N>(cu.n)), c(cu) {}
+  __device__ __forceinline__ R Pr(int p) const { return win[p * 32]; }
   // links are asked for the unit's own sites only
   __device__ __forceinline__ int Upr(int j) const { return j == c.a ? c.ua : c.ub; }
   __device__ __forceinline__ int Dnr(int j) const { return j == c.a ? c.da : c.db; }
   __device__ __forceinline__ R Njr(int j) const { return j == c.a ? c.na : c.nb; }
-  __device__ __forceinline__ R Gr(int p, int h) const { return base[p * Mp + h]; }
-  __device__ __forceinline__ R Yr(int p) const { return y[p * Mp]; }
-  __device__ __forceinline__ void Str(int p, R v) const { wout[p * Mp] = v; }
+  __device__ __forceinline__ R Gr(int p, int h) const { return base[node_col<N>(h) + p * 32]; }
+  __device__ __forceinline__ R Yr(int p) const { return y[p * 32]; }
+  __device__ __forceinline__ void Str(int p, R v) const { wout[p * 32] = v; }
 };
 
 template <int N, typename R>
@@ -1260,7 +1103,7 @@ __device__ __forceinline__ void write_row0(const Inst& I) {
   if (I.out_pops)
     for (int a = 0; a < N; ++a)
       I.out_pops[a] = MIXED ? ff_to_double(static_cast<const FF*>(I.y0)[a * N + a])
-                            : (double)static_cast<const R*>(I.y)[(a * N + a) * I.Mpad];
+                            : (double)static_cast<const R*>(I.y)[(a * N + a) * I.rstride];
   if (I.out_el) {
     I.out_el[0] = I.acc[0];
     I.out_el[1] = I.acc[1];
@@ -1326,8 +1169,9 @@ struct EtaRows {
 // The stop rule: true when the site population of the root after the step
 // just finished is below I.stop_trace.  Every CTA of the team evaluates it
 // from the same memory after the stage barrier, so all take the same branch.
+// dstep: distance of the root's diagonal elements in y's order (0: packed order, N + 1).
 template <typename R, bool MIXED>
-__device__ __forceinline__ bool stop_now(const Inst& I, int N, int* s_flag) {
+__device__ __forceinline__ bool stop_now(const Inst& I, int N, int* s_flag, int dstep = 0) {
   if (threadIdx.x == 0) {
     double tr = 0.0;
     if constexpr (MIXED) {
@@ -1337,7 +1181,8 @@ __device__ __forceinline__ bool stop_now(const Inst& I, int N, int* s_flag) {
       tr = ff_to_double(sum);
     } else {
       const R* y = static_cast<const R*>(I.y);
-      for (int a = 0; a < N; ++a) tr += (double)__ldcg(y + (size_t)(a * N + a) * I.Mpad);
+      if (dstep == 0) dstep = N + 1;
+      for (int a = 0; a < N; ++a) tr += (double)__ldcg(y + (size_t)(a * dstep) * I.rstride);
     }
     *s_flag = tr < I.stop_trace;
   }
@@ -1359,7 +1204,7 @@ __device__ __forceinline__ void finish_instance(const Inst& I, int nslots, const
       const float* y0 = static_cast<const float*>(I.y0);
       flag_nonfinite(status, (double)__ldcg(y0 + 2 * (a * N + a)) + (double)__ldcg(y0 + 2 * (a * N + a) + 1));
     } else {
-      flag_nonfinite(status, (double)__ldcg(static_cast<const R*>(I.y) + (size_t)(a * N + a) * I.Mpad));
+      flag_nonfinite(status, (double)__ldcg(static_cast<const R*>(I.y) + (size_t)(a * N + a) * I.rstride));
     }
   }
   if (done < I.nsteps) {
@@ -1389,23 +1234,10 @@ __device__ __forceinline__ void finish_instance(const Inst& I, int nslots, const
 
 // ------------------------------------------------------ global-memory engine
 
-// Dynamic shared memory of the global engine: with FP32 register views (unit
-// groups G <= 2, many units per item) the output staging of every warp,
-// [N*N][32] floats each; none otherwise.
-__host__ __device__ constexpr int engine_dyn_bytes(int N, int block, int rsize, bool reg) {
-  return (reg && rsize == 4) ? (block / 32) * N * N * 32 * rsize : 0;
-}
-
-// SC: scaled hierarchy (link weights from Inst::wsc); not with the FP32
-// register view, whose branch-free units take no weights.
-template <int N, typename R, bool MIXED, bool CPLX, bool REG, bool SC = false>
-__global__ void __launch_bounds__(sizeof(R) == 8 ? 256 : 512, (sizeof(R) == 8 && !REG) ? 2 : 1)
-    heom_engine_kernel(EngineArgs A) {
-  static_assert(!(SC && REG && sizeof(R) == 4), "no scaled FP32 register view");
-  extern __shared__ __align__(16) unsigned char dsm[];
+// SC: scaled hierarchy (link weights from Inst::wsc).
+template <int N, typename R, bool MIXED, bool CPLX, bool SC = false>
+__global__ void __launch_bounds__(sizeof(R) == 8 ? 256 : 512, sizeof(R) == 8 ? 2 : 1) heom_engine_kernel(EngineArgs A) {
   __shared__ __align__(16) unsigned char s_coef[CoefLayout<R>::bytes(kMaxSmallN) + 64];
-  __shared__ FF s_rootff[kMaxSmallN * kMaxSmallN];
-  __shared__ double s_pops[kMaxSmallN];
   __shared__ Inst s_inst;
   __shared__ int s_stop;
   __shared__ uint64_t s_umask[32];
@@ -1454,7 +1286,6 @@ __global__ void __launch_bounds__(sizeof(R) == 8 ? 256 : 512, (sizeof(R) == 8 &&
   const bool lead = (warp == 0 && lane == 0);
   const int nslots = G < 32 ? G : 32;
   unsigned epoch = 0;
-  const Staging<R> sg{reinterpret_cast<R*>(dsm) + (threadIdx.x >> 5) * (N * N * 32) + lane, s_rootff, s_pops};
 
   for (int li = A.team_first[team]; li < A.team_first[team + 1]; ++li) {
     load_instance<R>(A, li, s_inst, s_coef);
@@ -1476,7 +1307,7 @@ __global__ void __launch_bounds__(sizeof(R) == 8 ? 256 : 512, (sizeof(R) == 8 &&
 
     R* arr[3] = {static_cast<R*>(I.y), static_cast<R*>(I.wa), static_cast<R*>(I.wb)};
     // FP32 load views with one unit per warp: the unit and its links stay in registers
-    constexpr bool CACHE_OK = !REG && sizeof(R) == 4;
+    constexpr bool CACHE_OK = sizeof(R) == 4;
     const bool cached = CACHE_OK && G >= N * (N + 1) / 2 && items <= W;
     CachedUnit<R> cu;
     if (CACHE_OK && cached) cu = cache_unit<N, R>(I, warp, G, lane);
@@ -1507,31 +1338,12 @@ __global__ void __launch_bounds__(sizeof(R) == 8 ? 256 : 512, (sizeof(R) == 8 &&
           const int g = it - nb * G;
           const int n = (nb << 5) + lane;
           if (n >= I.M) continue;
-          const GlobalView<N, R, REG> v(ga, n);
+          const GlobalView<N, R> v(ga, n);
           const R ng = ngam[n];
-          // FP32 register views: staged, branch-free units (see unit_rhs), and the
-          // root's code only in the items that hold it.  Other views run one
-          // instantiation for every item (measured faster: a second copy of the
-          // unit code costs more in instruction fetch than the root branches).
-          constexpr bool BF = REG && sizeof(R) == 4;
-          if constexpr (!REG && sizeof(R) == 4) {
+          if constexpr (sizeof(R) == 4)
             node_units_rt<N, R, MIXED, CPLX, SC>(I, cf, cfd, P, v, ng, s, n == 0, s_umask[g], os, ea);
-          } else if constexpr (!BF) {
-            node_units<N, R, MIXED, CPLX, 0, 0, true, false, false, SC>(I, cf, cfd, P, v, ng, s, n == 0,
-                                                                        s_umask[g], os, ea, sg);
-          } else if (nb == 0) {
-            node_units<N, R, MIXED, CPLX, 0, 0, true, true, true, false>(I, cf, cfd, P, v, ng, s, n == 0,
-                                                                         s_umask[g], os, ea, sg);
-          } else if (G == 1) {
-            node_units<N, R, MIXED, CPLX, 1, 0, false, true, true, false>(I, cf, cfd, P, v, ng, s, false, 0, os, ea,
-                                                                          sg);
-          } else if (g == 0) {  // G == 2
-            node_units<N, R, MIXED, CPLX, 2, 0, false, true, true, false>(I, cf, cfd, P, v, ng, s, false, 0, os, ea,
-                                                                          sg);
-          } else {
-            node_units<N, R, MIXED, CPLX, 2, 1, false, true, true, false>(I, cf, cfd, P, v, ng, s, false, 0, os, ea,
-                                                                          sg);
-          }
+          else
+            node_units<N, R, MIXED, CPLX, SC>(I, cf, cfd, P, v, ng, s, n == 0, s_umask[g], os, ea);
         }
         if (s == 2 && slot >= 0) ea.step_xi(I);
         if (s == 3 && slot >= 0 && (os.now || t + 1 == I.nsteps)) ea.store(I, slot);
@@ -1627,7 +1439,7 @@ __global__ void __launch_bounds__(512) heom_smem_kernel(EngineArgs A, int B) {
     const float* gy = static_cast<const float*>(I.y);
     for (int idx = threadIdx.x; idx < NN * B; idx += blockDim.x) {
       const int p = idx / B, l = idx - (idx / B) * B;
-      sy[idx] = l < nloc ? gy[p * Mp + n0 + l] : 0.f;
+      sy[idx] = l < nloc ? gy[node_col<N>(n0 + l) + p * 32] : 0.f;
     }
     for (int idx = threadIdx.x; idx < N * B; idx += blockDim.x) {
       const int j = idx / B, l = idx - (idx / B) * B;
@@ -1685,9 +1497,7 @@ __global__ void __launch_bounds__(512) heom_smem_kernel(EngineArgs A, int B) {
           const int l = (nb << 5) + lane;
           if (l >= nloc) continue;
           const SmemView<N, REG> v(sa, l);
-          node_units<N, float, true, CPLX, 0, 0, true, false, false, false>(I, cf, cfd, P, v, sng[l], s, rank == 0 && l == 0,
-                                                                     s_umask[g], os, ea,
-                                                                     Staging<float>{nullptr, nullptr, nullptr});
+          node_units<N, float, true, CPLX, false>(I, cf, cfd, P, v, sng[l], s, rank == 0 && l == 0, s_umask[g], os, ea);
         }
         if (s == 2 && slot >= 0) ea.step_xi(I);
         if (s == 3 && slot >= 0 && (os.now || t + 1 == I.nsteps)) ea.store(I, slot);
@@ -1706,7 +1516,7 @@ __global__ void __launch_bounds__(512) heom_smem_kernel(EngineArgs A, int B) {
     float* gyw = static_cast<float*>(I.y);
     for (int idx = threadIdx.x; idx < NN * B; idx += blockDim.x) {
       const int p = idx / B, l = idx - (idx / B) * B;
-      if (l < nloc) gyw[p * Mp + n0 + l] = sy[idx];
+      if (l < nloc) gyw[node_col<N>(n0 + l) + p * 32] = sy[idx];
     }
     cluster_sync_all();  // no CTA reuses or leaves its slice while others may still read it
     if (lead) signal_done(I);

@@ -57,7 +57,9 @@ constexpr int kFlowMaxThreads = 384;
 // registers (with ten or twelve warps some sub-partition holds three, and its
 // register file allows 168).
 constexpr int kFlowMaxThreadsMulti = 256;
-constexpr int kFlowMaxNpt = 6;
+constexpr int kFlowMaxNpt = 6;       // accepted by the launch shape
+// built; more nodes per thread run the throughput engine (see launch_flow)
+__host__ __device__ constexpr int flow_built_npt(int N) { return N == 8 ? 2 : 3; }
 
 // One unit's own-node linear form (host-built).  Slot 0 of both lists is the
 // unit's own real element x = P[a*N + b]; for a pair, slot 1 is its imaginary
@@ -334,8 +336,8 @@ __global__ void __launch_bounds__(NPT == 1 ? kFlowMaxThreads : kFlowMaxThreadsMu
     y_r[k] = y_i[k] = R(0);
     if (!valid[k]) continue;
     const int oab = pab * Mp + nd[k], oba = pba * Mp + nd[k];
-    y_r[k] = gy[oab];
-    y_i[k] = pair ? gy[oba] : R(0);
+    y_r[k] = gy[node_col<N>(nd[k]) + pab * 32];
+    y_i[k] = pair ? gy[node_col<N>(nd[k]) + pba * 32] : R(0);
     R* own = sb + (k * S + l) * NN;
     own[pab] = y_r[k];
     if (pair) own[pba] = y_i[k];
@@ -575,13 +577,13 @@ __global__ void __launch_bounds__(NPT == 1 ? kFlowMaxThreads : kFlowMaxThreadsMu
       }
     }
   }
-  // the state back to device memory (packed, element-major; the root also in float-float)
+  // the state back to device memory (packed, see node_col; the root also in float-float)
   R* gyw = static_cast<R*>(I.y);
 #pragma unroll
   for (int k = 0; k < NPT; ++k) {
     if (!valid[k]) continue;
-    gyw[pab * Mp + nd[k]] = y_r[k];
-    if (pair) gyw[pba * Mp + nd[k]] = y_i[k];
+    gyw[node_col<N>(nd[k]) + pab * 32] = y_r[k];
+    if (pair) gyw[node_col<N>(nd[k]) + pba * 32] = y_i[k];
   }
   if constexpr (MIXED) {
     if (root) {

@@ -6,13 +6,17 @@
 
 namespace heom {
 
-// Engine kernel entry points for N = 1..8 (nullptr otherwise); reg selects
-// the register-resident node view.
-const void* engine_kernel_f64_real(int N, bool reg);
-const void* engine_kernel_f64_cplx(int N, bool reg);
-const void* engine_kernel_f32_real(int N, bool reg);
-const void* engine_kernel_f32_cplx(int N, bool reg);
-// Scaled hierarchies (HEOM_FLAG_SCALED), N = 1..8, load views only.
+// Load-view engine for N = 1..8 (nullptr otherwise): any number of unit groups.
+const void* engine_kernel_f64_real(int N);
+const void* engine_kernel_f64_cplx(int N);
+const void* engine_kernel_f32_real(int N);
+const void* engine_kernel_f32_cplx(int N);
+// Throughput engine for N = 1..8 (nullptr otherwise), scaled hierarchies included.
+const void* block_kernel_f64_real(int N);
+const void* block_kernel_f64_cplx(int N);
+const void* block_kernel_f32_real(int N);
+const void* block_kernel_f32_cplx(int N);
+// Scaled hierarchies (HEOM_FLAG_SCALED), N = 1..8, load views.
 const void* engine_kernel_scaled_f64(int N, bool cplx);
 const void* engine_kernel_scaled_f32(int N, bool cplx);
 // Large-N engine (9..24 sites).
@@ -30,14 +34,19 @@ const void* smem_kernel_f32_cplx(int N, bool reg);
 inline const void* smem_kernel(bool cplx, bool reg, int N) {
   return cplx ? smem_kernel_f32_cplx(N, reg) : smem_kernel_f32_real(N, reg);
 }
-// nullptr where there is no such kernel (N > 8, or a scaled register view)
-inline const void* engine_kernel(bool fp64, bool cplx, bool reg, int N, bool scaled = false) {
-  if (scaled) {
-    if (reg) return nullptr;
-    return fp64 ? engine_kernel_scaled_f64(N, cplx) : engine_kernel_scaled_f32(N, cplx);
-  }
-  if (fp64) return cplx ? engine_kernel_f64_cplx(N, reg) : engine_kernel_f64_real(N, reg);
-  return cplx ? engine_kernel_f32_cplx(N, reg) : engine_kernel_f32_real(N, reg);
+inline const void* block_kernel(bool fp64, bool cplx, int N) {
+  if (fp64) return cplx ? block_kernel_f64_cplx(N) : block_kernel_f64_real(N);
+  return cplx ? block_kernel_f32_cplx(N) : block_kernel_f32_real(N);
+}
+// Kernel of launch modes 0 and 1 for node_threads G: the throughput engine for
+// 1, 2 and 4, the load views otherwise; scaled hierarchies refuse 1 and 2.
+// nullptr where there is no such kernel.
+inline const void* engine_kernel(bool fp64, bool cplx, int G, int N, bool scaled = false) {
+  if (scaled && G <= 2) return nullptr;
+  if (G == 1 || G == 2 || G == 4) return block_kernel(fp64, cplx, N);
+  if (scaled) return fp64 ? engine_kernel_scaled_f64(N, cplx) : engine_kernel_scaled_f32(N, cplx);
+  if (fp64) return cplx ? engine_kernel_f64_cplx(N) : engine_kernel_f64_real(N);
+  return cplx ? engine_kernel_f32_cplx(N) : engine_kernel_f32_real(N);
 }
 
 // Hierarchy index builder (heom_index.cpp).

@@ -5,27 +5,18 @@
 
 namespace heom {
 
-const void* engine_kernel_f32_cplx(int N, bool reg) {
+const void* engine_kernel_f32_cplx(int N) {
   switch (N) {
-    case 1: return reg ? (const void*)heom_engine_kernel<1, float, true, true, true>
-                    : (const void*)heom_engine_kernel<1, float, true, true, false>;
-    case 2: return reg ? (const void*)heom_engine_kernel<2, float, true, true, true>
-                    : (const void*)heom_engine_kernel<2, float, true, true, false>;
-    case 3: return reg ? (const void*)heom_engine_kernel<3, float, true, true, true>
-                    : (const void*)heom_engine_kernel<3, float, true, true, false>;
-    case 4: return reg ? (const void*)heom_engine_kernel<4, float, true, true, true>
-                    : (const void*)heom_engine_kernel<4, float, true, true, false>;
-    case 5: return reg ? (const void*)heom_engine_kernel<5, float, true, true, true>
-                    : (const void*)heom_engine_kernel<5, float, true, true, false>;
-    case 6: return reg ? (const void*)heom_engine_kernel<6, float, true, true, true>
-                    : (const void*)heom_engine_kernel<6, float, true, true, false>;
-    case 7: return reg ? (const void*)heom_engine_kernel<7, float, true, true, true>
-                    : (const void*)heom_engine_kernel<7, float, true, true, false>;
-    case 8: return reg ? (const void*)heom_engine_kernel<8, float, true, true, true>
-                    : (const void*)heom_engine_kernel<8, float, true, true, false>;
+    case 1: return (const void*)heom_engine_kernel<1, float, true, true>;
+    case 2: return (const void*)heom_engine_kernel<2, float, true, true>;
+    case 3: return (const void*)heom_engine_kernel<3, float, true, true>;
+    case 4: return (const void*)heom_engine_kernel<4, float, true, true>;
+    case 5: return (const void*)heom_engine_kernel<5, float, true, true>;
+    case 6: return (const void*)heom_engine_kernel<6, float, true, true>;
+    case 7: return (const void*)heom_engine_kernel<7, float, true, true>;
+    case 8: return (const void*)heom_engine_kernel<8, float, true, true>;
     default: return nullptr;
   }
 }
-
 
 }  // namespace heom

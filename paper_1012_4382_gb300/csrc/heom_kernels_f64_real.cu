@@ -5,24 +5,16 @@
 
 namespace heom {
 
-const void* engine_kernel_f64_real(int N, bool reg) {
+const void* engine_kernel_f64_real(int N) {
   switch (N) {
-    case 1: return reg ? (const void*)heom_engine_kernel<1, double, false, false, true>
-                    : (const void*)heom_engine_kernel<1, double, false, false, false>;
-    case 2: return reg ? (const void*)heom_engine_kernel<2, double, false, false, true>
-                    : (const void*)heom_engine_kernel<2, double, false, false, false>;
-    case 3: return reg ? (const void*)heom_engine_kernel<3, double, false, false, true>
-                    : (const void*)heom_engine_kernel<3, double, false, false, false>;
-    case 4: return reg ? (const void*)heom_engine_kernel<4, double, false, false, true>
-                    : (const void*)heom_engine_kernel<4, double, false, false, false>;
-    case 5: return reg ? (const void*)heom_engine_kernel<5, double, false, false, true>
-                    : (const void*)heom_engine_kernel<5, double, false, false, false>;
-    case 6: return reg ? (const void*)heom_engine_kernel<6, double, false, false, true>
-                    : (const void*)heom_engine_kernel<6, double, false, false, false>;
-    case 7: return reg ? (const void*)heom_engine_kernel<7, double, false, false, true>
-                    : (const void*)heom_engine_kernel<7, double, false, false, false>;
-    case 8: return reg ? (const void*)heom_engine_kernel<8, double, false, false, true>
-                    : (const void*)heom_engine_kernel<8, double, false, false, false>;
+    case 1: return (const void*)heom_engine_kernel<1, double, false, false>;
+    case 2: return (const void*)heom_engine_kernel<2, double, false, false>;
+    case 3: return (const void*)heom_engine_kernel<3, double, false, false>;
+    case 4: return (const void*)heom_engine_kernel<4, double, false, false>;
+    case 5: return (const void*)heom_engine_kernel<5, double, false, false>;
+    case 6: return (const void*)heom_engine_kernel<6, double, false, false>;
+    case 7: return (const void*)heom_engine_kernel<7, double, false, false>;
+    case 8: return (const void*)heom_engine_kernel<8, double, false, false>;
     default: return nullptr;
   }
 }

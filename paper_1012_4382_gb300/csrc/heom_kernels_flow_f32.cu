@@ -1,6 +1,6 @@
 // Instantiations of the dataflow engine (launch mode 3) for N = 1..8, mixed precision (float auxiliaries, float-float root).
-// One node per thread for every N and H; with real H and N >= 4 also 2 to 6
-// nodes per thread (hierarchies too large for one node per thread).
+// One node per thread for every N and H; with real H and N >= 4 also 2 and (N <= 7)
+// 3 nodes per thread (hierarchies too large for one node per thread).
 // (One translation unit per precision so they compile in parallel.)
 #include "heom_flow.cuh"
 #include "heom_internal.h"
@@ -16,10 +16,9 @@ const void* flow_pick(bool cplx, int npt) {
     if (cplx) return nullptr;
     switch (npt) {
       case 2: return (const void*)heom_flow_kernel<N, R, MIXED, false, 2>;
-      case 3: return (const void*)heom_flow_kernel<N, R, MIXED, false, 3>;
-      case 4: return (const void*)heom_flow_kernel<N, R, MIXED, false, 4>;
-      case 5: return (const void*)heom_flow_kernel<N, R, MIXED, false, 5>;
-      case 6: return (const void*)heom_flow_kernel<N, R, MIXED, false, 6>;
+      case 3:
+        if constexpr (flow_built_npt(N) >= 3) return (const void*)heom_flow_kernel<N, R, MIXED, false, 3>;
+        return nullptr;
       default: return nullptr;
     }
   }

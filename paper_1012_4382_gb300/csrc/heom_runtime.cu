@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "heom.h"
+#include "heom_block.cuh"
 #include "heom_flow.cuh"
 #include "heom_large.cuh"
 #include "heom_internal.h"
@@ -188,14 +189,14 @@ __global__ void set_root_kernel(R* y, int Mpad, float2* y0, const double* rho, i
       v = rho[2 * (b * N + a) + 1];
     else
       v = rho[2 * (a * N + a)];
-    y[(size_t)p * Mpad] = (R)v;
+    y[heom::state_elem(N, Mpad, p, 0)] = (R)v;
     if (y0) y0[p] = to_ff(v);
   }
   if (p == 0)
     for (int k = 0; k < kAccDoubles; ++k) acc[k] = 0.0;
 }
 
-// packed element-major state -> full complex matrices [M][N][N]
+// packed state -> full complex matrices [M][N][N]
 template <typename R>
 __global__ void unpack_state_kernel(const R* y, int Mpad, int64_t M, int N, const float2* y0, double* out) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -206,7 +207,7 @@ __global__ void unpack_state_kernel(const R* y, int Mpad, int64_t M, int N, cons
   const int a = e / N, b = e - (e / N) * N;
   auto P = [&](int k, int l) -> double {
     if (n == 0 && y0) return (double)y0[k * N + l].x + (double)y0[k * N + l].y;
-    return (double)y[(size_t)(k * N + l) * Mpad + n];
+    return (double)y[heom::state_elem(N, Mpad, k * N + l, n)];
   };
   double re, im;
   if (a < b) {
@@ -239,13 +240,13 @@ __global__ void pack_state_kernel(const double* in, R* y, int Mpad, int64_t M, i
     v = m[2 * (b * N + a) + 1];
   else
     v = m[2 * (a * N + a)];
-  y[(size_t)p * Mpad + n] = (R)v;
+  y[heom::state_elem(N, Mpad, p, n)] = (R)v;
   if (n == 0 && y0) y0[p] = to_ff(v);
 }
 
 int launch_blocks(int64_t work, int threads) { return (int)((work + threads - 1) / threads); }
 
-// Largest element modulus of every node's matrix (packed, element-major):
+// Largest element modulus of every node's matrix (packed):
 // out[n] = max_ab |sigma_n,ab|, one thread per node.
 template <typename R>
 __global__ void node_max_kernel(const R* y, int Mpad, int64_t M, int N, double* out) {
@@ -253,9 +254,10 @@ __global__ void node_max_kernel(const R* y, int Mpad, int64_t M, int N, double* 
   if (n >= M) return;
   double mx = 0.0;
   for (int a = 0; a < N; ++a) {
-    mx = fmax(mx, fabs((double)y[(size_t)(a * N + a) * Mpad + n]));
+    mx = fmax(mx, fabs((double)y[heom::state_elem(N, Mpad, a * N + a, n)]));
     for (int b = a + 1; b < N; ++b) {
-      const double re = (double)y[(size_t)(a * N + b) * Mpad + n], im = (double)y[(size_t)(b * N + a) * Mpad + n];
+      const double re = (double)y[heom::state_elem(N, Mpad, a * N + b, n)];
+      const double im = (double)y[heom::state_elem(N, Mpad, b * N + a, n)];
       mx = fmax(mx, sqrt(re * re + im * im));
     }
   }
@@ -263,7 +265,7 @@ __global__ void node_max_kernel(const R* y, int Mpad, int64_t M, int N, double* 
 }
 
 // Device-side bounds and consistency check of a node table pair ([N][Mpad]
-// int32, element-major like the state; dn packs n_j in its top byte), run on
+// int32, node index innermost; dn packs n_j in its top byte), run on
 // the tables every kernel will read, before any propagation reads them.  For
 // node n < M and site j: an up link is -1 or a later node u < M whose down
 // link on site j is n with n_j(u) = n_j(n) + 1; a down link is -1 or an
@@ -777,18 +779,50 @@ struct Engine {
   }
 
   // Default launch shape for the instances with N sites.  Scaled hierarchies
-  // (N <= 8) need a load view (node_threads >= 3) in mode 0 or 1: where any
-  // instance of this N is scaled the plain default is moved there.
+  // (N <= 8) need node_threads >= 3 in mode 0 or 1: where any instance of this N
+  // is scaled the plain default is moved there (4: the throughput engine).
   LaunchCfg default_cfg(int N, int count) const {
     LaunchCfg c = default_cfg_plain(N, count);
     bool sc = false;
     for (auto& in : inst) sc |= (in->N == N && in->scaled);
     if (sc && N <= heom::kMaxSmallN) {
       if (c.mode == 2) c.mode = 0;
-      const int U = N * (N + 1) / 2;
-      if (c.G <= 2) c.G = std::max(3, std::min(8, U));
+      if (c.G <= 2) c.G = 4;
     }
     return c;
+  }
+
+  // CTAs per team for a batch's instances with N sites: of 1, 2, 4, 8 and 16 the one whose longest-first packing of
+  // the instances onto the teams the GPU holds at once has the shortest makespan, with a stage of b node blocks per
+  // CTA taking a + m b.  Measured (us, N = 7): a = 1.5; m = 0.52 in mixed precision, 8.1 in FP64 (the FP64 pipe);
+  // m scales about as N^2.5 (N = 5: 0.25 and 3.5, N = 8: 0.73 and 12).  Per step, team sizes 1, 2, 4, 8, 16: 256 mixed
+  // instances of depth 4 to 8 543, 398, 408, 411 us (2 picked); 24 FP64 ones of depth 4 to 7 -, 1745, 884, 463, 366
+  // (16 picked; 1745 with the former fixed 2); 30 mixed of depth 7 231, 121, 64, 73, 108 (4 picked).
+  int batch_team(int N) const {
+    std::vector<int64_t> blocks;
+    for (auto& in : inst)
+      if (in->N == N) blocks.push_back((in->M + 31) / 32);
+    std::sort(blocks.begin(), blocks.end(), std::greater<int64_t>());
+    const double m = (prec == HEOM_FP64 ? 8.1 : 0.52) * std::pow(N / 7.0, 2.5);
+    int best = 1;
+    double best_t = 0.0;
+    for (int c = 1; c <= 16; c *= 2) {
+      const size_t teams = std::min<size_t>(blocks.size(), std::max(1, sms / c));
+      std::priority_queue<double, std::vector<double>, std::greater<double>> load;
+      for (size_t t = 0; t < teams; ++t) load.push(0.0);
+      double span = 0.0;
+      for (int64_t b : blocks) {
+        const double t = load.top() + 1.5 + m * (double)((b + c - 1) / c);
+        load.pop();
+        load.push(t);
+        span = std::max(span, t);
+      }
+      if (c == 1 || span < 0.98 * best_t) {
+        best = c;
+        best_t = span;
+      }
+    }
+    return best;
   }
 
   LaunchCfg default_cfg_plain(int N, int count) const {
@@ -816,7 +850,8 @@ struct Engine {
       // over all SMs, S = ceil(M / SMs)
       // Beyond what one node per thread holds (about 1976 nodes at N = 7), each thread
       // carries npt = 2..6 nodes of its unit (real H, N >= 4; CTAs of at most 256 threads,
-      // the nodes spread evenly): the fewest nodes per thread with which all CTAs fit.
+      // the nodes spread evenly): the fewest nodes per thread with which all CTAs fit
+      // (launch_flow says what runs with more than three).
       if (Mmax >= 256) {
         const int U = N * (N + 1) / 2;
         bool cplx_any = false;
@@ -826,7 +861,7 @@ struct Engine {
           const int64_t even = (Mmax + (int64_t)sms * npt - 1) / ((int64_t)sms * npt);
           const int S = (int)std::min<int64_t>(
               maxthr / U, npt > 1 ? even : (prec == HEOM_FP64 ? even : std::max<int64_t>(336 / U, even)));
-          const void* k = heom::flow_kernel(prec == HEOM_FP64, cplx_any, N, npt);
+          const void* k = flow_kernel_shape(cplx_any, N, npt);
           if (S < 1 || !k) continue;
           const int dyn = heom::flow_smem_bytes(N, S * npt, (int)rsize());
           int per_sm = 0;
@@ -843,57 +878,30 @@ struct Engine {
         }
       }
       if ((prec == HEOM_FP64 && Mmax >= 256) || (prec == HEOM_FP32_MIXED && Mmax >= 1024)) {
-        // the grid engine: unit groups and CTA size as the autotuner picks them for the
-        // N = 7 trap hierarchies of depth 8, 10 and 12 (6435, 19448, 50388 nodes; 202, 608
-        // and 1575 blocks of 32 nodes): load views of 8 groups while the node blocks are
-        // few, the register view (2 groups) once they fill the GPU.  Measured against 32
-        // groups, 1000 steps: mixed 38.9 / 66.8 / 87.1 ms instead of 40.2 / 95.5 / 236.8,
-        // FP64 76.4 / 184.8 / 481 instead of 93.2 / 246.5 / 621
-        const int64_t nb = (Mmax + 31) / 32;
+        // the throughput engine on the whole grid
         c.mode = 1;
         c.team_ctas = 1;
-        if (N < 4) {
-          c.block = max_block();
-          c.G = 2;
-        } else if (prec == HEOM_FP64) {
-          c.G = nb < 400 ? 8 : 2;
-          c.block = nb < 1000 ? 128 : 256;
-        } else {
-          c.G = nb < 1000 ? 8 : 2;
-          c.block = c.G == 8 ? 512 : 256;
-        }
+        c.block = max_block();
+        c.G = 2;
       } else {
+        // small: the throughput engine in one CTA while its blocks of 32 nodes fill at most one round of sets, else
+        // in a cluster with a block per CTA
         c.mode = 0;
-        c.block = 256;
-        c.G = N >= 4 ? 8 : 2;
-        const int64_t units = ((Mmax + 31) / 32) * c.G;
-        const int64_t warps = c.block / 32;
-        int ctas = (int)std::min<int64_t>(16, std::max<int64_t>(1, (units + warps - 1) / warps));
-        int p2 = 1;
-        while (p2 < ctas) p2 <<= 1;
-        c.team_ctas = std::min(16, p2);
-        if (prec == HEOM_FP32_MIXED) {
-          // the hierarchy in the cluster's shared memory, ~128 nodes per CTA
-          int ct = 1;
-          while (ct < 16 && (ct * 128 < Mmax || heom::smem_dyn_bytes(N, smem_slice(Mmax, ct)) > max_dyn_smem())) ct <<= 1;
-          if (heom::smem_dyn_bytes(N, smem_slice(Mmax, ct)) <= max_dyn_smem()) {
-            c.mode = 2;
-            c.team_ctas = ct;
-            c.block = 512;
-            c.G = 4;
-          }
-        }
+        c.block = max_block();
+        c.G = 2;
+        const int64_t nb = (Mmax + 31) / 32;
+        c.team_ctas = 1;
+        if (nb > heom::block_sets(N, (int)rsize(), c.block))
+          while (c.team_ctas < 16 && c.team_ctas < nb) c.team_ctas <<= 1;
       }
     } else {
-      // many hierarchies: small teams so that every instance runs at once
+      // many hierarchies: the throughput engine with the team size batch_team picks.  Keeping small hierarchies in
+      // shared memory (mode 2) loses to it: 64 hierarchies of 70 nodes (N = 4) 14.9 us a step against 7.2, 300 of 252
+      // nodes (N = 5) 51 against 27
       c.mode = 0;
       c.block = max_block();
       c.G = 2;
-      c.team_ctas = 2;
-      if (prec == HEOM_FP32_MIXED && heom::smem_dyn_bytes(N, smem_slice(Mmax, 1)) <= max_dyn_smem()) {
-        c.mode = 2;
-        c.team_ctas = 1;
-      }
+      c.team_ctas = batch_team(N);
     }
     return c;
   }
@@ -964,7 +972,7 @@ struct Engine {
       CUDA_TRY(cudaMemcpyAsync(in->ngam.p, ng.data(), ng.size(), cudaMemcpyHostToDevice, stream));
       CUDA_TRY(cudaStreamSynchronize(stream));
     }
-    const size_t arr = (size_t)p.N * p.N * in->Mpad * rsize();
+    const size_t arr = heom::state_reals(p.N, in->Mpad) * rsize();
     TRY(in->y.alloc(arr, hooks));
     TRY(in->wa.alloc(arr, hooks));
     TRY(in->wb.alloc(arr, hooks));
@@ -975,6 +983,11 @@ struct Engine {
     TRY(in->stage.alloc(2 * sizeof(double) * p.N * p.N, hooks));
     CUDA_TRY(cudaMemcpyAsync(in->coef.p, in->coef_host.data(), in->coef_host.size(), cudaMemcpyHostToDevice, stream));
     CUDA_TRY(cudaMemsetAsync(in->y.p, 0, arr, stream));
+    if (p.N <= heom::kMaxSmallN) {  // the block of zeros that ends each stage buffer
+      const size_t live = (size_t)p.N * p.N * in->Mpad * rsize();
+      CUDA_TRY(cudaMemsetAsync(in->wa.as<unsigned char>() + live, 0, arr - live, stream));
+      CUDA_TRY(cudaMemsetAsync(in->wb.as<unsigned char>() + live, 0, arr - live, stream));
+    }
     CUDA_TRY(cudaMemsetAsync(in->acc.p, 0, kAccDoubles * sizeof(double), stream));
     CUDA_TRY(cudaStreamSynchronize(stream));  // coef_host must outlive the copy
     inst.push_back(std::move(in));
@@ -1038,7 +1051,7 @@ struct Engine {
 
   int set_rho0_device(int i, const double* d_rho) {
     Instance& in = *inst[i];
-    const size_t arr = (size_t)in.N * in.N * in.Mpad * rsize();
+    const size_t arr = heom::state_reals(in.N, in.Mpad) * rsize();
     CUDA_TRY(cudaMemsetAsync(in.y.p, 0, arr, stream));
     const int NN = in.N * in.N;
     if (prec == HEOM_FP64)
@@ -1081,6 +1094,7 @@ struct Engine {
       d.K = in.K;
       d.M = (int32_t)in.M;
       d.Mpad = in.Mpad;
+      d.rstride = in.N <= heom::kMaxSmallN ? 32 : in.Mpad;
       d.complex_h = in.complex_h;
       d.terminator = in.terminator;
       d.up = in.tab->up.as<int32_t>();
@@ -1152,8 +1166,10 @@ struct Engine {
                       "launch mode 2: %lld nodes of N=%d need %d bytes of shared memory per CTA with %d CTAs "
                       "(at most %d); use more team CTAs or mode 0",
                       (long long)Mmax, g.N, g.dyn, g.c.team_ctas, max_dyn_smem());
-      } else {
-        g.dyn = heom::engine_dyn_bytes(g.N, g.c.block, (int)rsize(), g.c.G <= 2);
+      } else if (block_engine(g.N, g.sc, g.c)) {
+        int64_t Mmax = 0;
+        for (int id : ids) Mmax = std::max<int64_t>(Mmax, inst[id]->M);
+        block_shape(g.N, g.c, Mmax, &g.B, &g.dyn);
       }
       if (!kernel_for(g.N, g.cplx, g.sc, g.c))
         return fail(HEOM_EUNSUPPORTED, "no engine kernel for N=%d, launch mode %d, node_threads %d%s", g.N, g.c.mode,
@@ -1285,7 +1301,7 @@ struct Engine {
       A.gsync = d_gsync.as<unsigned>();
       A.status = d_status.as<int>();
       if (g.c.mode == 3) {
-        TRY(launch_flow(*inst[g.list[0]], g.c, A.insts + g.list[0], A.status, nsteps[g.list[0]]));
+        TRY(launch_flow(*inst[g.list[0]], g.c, A, A.insts + g.list[0], nsteps[g.list[0]]));
         continue;
       }
       TRY(launch(g.N, g.cplx, g.sc, g.c, g.nteams, A, g.B, g.dyn));
@@ -1293,17 +1309,24 @@ struct Engine {
     return HEOM_OK;
   }
 
+  // The dataflow kernel that stands for npt nodes per thread: the built one, and for more (mixed precision) the largest built,
+  // which takes the same registers per thread and so has the same residency.  nullptr: not supported.
+  const void* flow_kernel_shape(bool cplx, int N, int npt) const {
+    if (N > heom::kMaxSmallN || npt < 1 || npt > heom::kFlowMaxNpt) return nullptr;
+    return heom::flow_kernel(prec == HEOM_FP64, cplx, N, std::min(npt, heom::flow_built_npt(N)));
+  }
+
   // Nodes per CTA of the dataflow engine for a block of `block` threads.
   static int flow_nodes_per_cta(int N, int block) { return std::max(1, block / (N * (N + 1) / 2)); }
 
   // The dataflow engine (mode 3) on one instance: the unit table and the
   // tagged stage buffers on first use, the tag base, one cooperative launch.
-  int launch_flow(Instance& in, const LaunchCfg& c, const Inst* d_inst, int* d_status, int64_t nsteps) {
+  int launch_flow(Instance& in, const LaunchCfg& c, EngineArgs& A, const Inst* d_inst, int64_t nsteps) {
     NvtxRange range("heom dataflow launch");
     const int N = in.N, U = N * (N + 1) / 2, NN = N * N;
     const bool fp64 = prec == HEOM_FP64;
     const int npt = c.team_ctas;  // nodes per thread
-    const void* k = heom::flow_kernel(fp64, in.complex_h != 0, N, npt);
+    const void* k = flow_kernel_shape(in.complex_h != 0, N, npt);
     if (!k)
       return fail(HEOM_EUNSUPPORTED,
                   "launch mode 3 takes at most %d sites, and more than one node per thread only with real H "
@@ -1317,6 +1340,29 @@ struct Engine {
     const int SL = S * npt;  // nodes of a CTA's slice
     const int grid = (int)((in.M + SL - 1) / SL);
     const int dyn = heom::flow_smem_bytes(N, SL, (int)rsize());
+    CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+    int per_sm = 0;
+    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, dyn));
+    if ((int64_t)per_sm * sms < grid)
+      return fail(HEOM_EINVAL,
+                  "launch mode 3: %d CTAs of %d nodes (%d threads) cannot all be resident (%d per SM); use "
+                  "more nodes per CTA or per thread, or another mode",
+                  grid, SL, threads, per_sm);
+    if (npt > heom::flow_built_npt(N)) {
+      // Four or more nodes per thread (three or more at N = 8): the throughput engine on the whole grid is faster than that many nodes' serial
+      // updates (us per step, N = 7 depth 8, five nodes per thread: 17.5 dataflow, 13.0; N = 6 depth 10: 19.0, 12.5;
+      // with three nodes per thread 9.1 dataflow, 12.0, but at N = 8 17.4, 13.3), so it runs in the dataflow kernel's
+      // place
+      LaunchCfg g;
+      g.mode = 1;
+      g.block = max_block();
+      g.G = 4;
+      A.mode = 1;
+      A.G = g.G;
+      int links = 0, bytes = 0;
+      block_shape(N, g, in.M, &links, &bytes);
+      return launch(N, in.complex_h, in.scaled, g, 1, A, links, bytes);
+    }
     const long long wd = fp64 ? 2 : 1;
     const long long stride = (long long)NN * in.Mpad * wd;
     if (!in.flow_tags.p) {
@@ -1334,21 +1380,13 @@ struct Engine {
       CUDA_TRY(cudaMemsetAsync(in.flow_tags.p, 0, in.flow_tags.bytes, stream));
       in.flow_tag = 0;
     }
-    CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-    int per_sm = 0;
-    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, dyn));
-    if ((int64_t)per_sm * sms < grid)
-      return fail(HEOM_EINVAL,
-                  "launch mode 3: %d CTAs of %d nodes (%d threads) cannot all be resident (%d per SM); use "
-                  "more nodes per CTA or per thread, or another mode",
-                  grid, SL, threads, per_sm);
     heom::FlowArgs F;
     F.inst = d_inst;
     F.units = in.flow_units.as<heom::FlowUnit>();
     F.tags = in.flow_tags.as<unsigned long long>();
     F.tag_stride = stride;
     F.ring = F.tags + 3 * stride;
-    F.status = d_status;
+    F.status = A.status;
     F.S = S;
     F.tag0 = in.flow_tag;
     in.flow_tag += need;
@@ -1358,18 +1396,40 @@ struct Engine {
   }
 
   // The kernel of a launch shape, or nullptr where none is built: mode 2 for
-  // FP64 or N > 8; scaled hierarchies in mode 2 or with the register view
-  // (node_threads <= 2) for N <= 8.
+  // FP64 or N > 8; scaled hierarchies in mode 2 or with node_threads <= 2 for
+  // N <= 8.
   const void* kernel_for(int N, int cplx, int sc, const LaunchCfg& c) const {
-    if (c.mode == 3)
-      return N > heom::kMaxSmallN ? nullptr : heom::flow_kernel(prec == HEOM_FP64, cplx != 0, N, c.team_ctas);
+    if (c.mode == 3) return flow_kernel_shape(cplx != 0, N, c.team_ctas);
     if (N > heom::kMaxSmallN) return c.mode == 2 ? nullptr : heom::large_kernel(prec == HEOM_FP64, cplx != 0, sc != 0);
     if (c.mode == 2) return (prec == HEOM_FP64 || sc) ? nullptr : heom::smem_kernel(cplx != 0, c.G <= 2, N);
-    return heom::engine_kernel(prec == HEOM_FP64, cplx != 0, c.G <= 2, N, sc != 0);
+    return heom::engine_kernel(prec == HEOM_FP64, cplx != 0, c.G, N, sc != 0);
   }
   static const char* no_kernel_reason(int N, int sc) {
     if (sc && N <= heom::kMaxSmallN) return " (scaled hierarchies take modes 0 and 1 with node_threads >= 3)";
     return "";
+  }
+
+  // Does this shape run the throughput engine (heom_block.cuh)?
+  static bool block_engine(int N, int sc, const LaunchCfg& c) {
+    return N <= heom::kMaxSmallN && c.mode <= 1 && (c.G == 4 || (!sc && (c.G == 1 || c.G == 2)));
+  }
+  // Throughput engine: the blocks whose links a CTA keeps in shared memory (all of its share of a hierarchy of M nodes
+  // when that takes at most 96 KB, which leaves the L1 its share; else none) and its dynamic shared memory.
+  void block_shape(int N, const LaunchCfg& c, int64_t M, int* link_cache, int* dyn) const {
+    const int ctas = c.mode == 1 ? sms : c.team_ctas;
+    const int64_t blocks = ((M + 31) / 32 + ctas - 1) / ctas;
+    *link_cache = blocks * heom::block_link_bytes(N) <= 96 * 1024 ? (int)blocks : 0;
+    *dyn = heom::block_exch_bytes(N, (int)rsize(), heom::block_sets(N, (int)rsize(), c.block)) +
+           *link_cache * heom::block_link_bytes(N);
+  }
+  int block_dyn(int N, const LaunchCfg& c, int64_t M) const {
+    int links = 0, dyn = 0;
+    block_shape(N, c, M, &links, &dyn);
+    return dyn;
+  }
+  // Threads per CTA of a launch of modes 0 to 2: the block asked for, or the throughput engine's sets for it.
+  int cta_threads(int N, int sc, const LaunchCfg& c) const {
+    return block_engine(N, sc, c) ? 32 * N * heom::block_sets(N, (int)rsize(), c.block) : c.block;
   }
 
   // Nodes per CTA when a cluster of `ctas` CTAs holds M nodes (mode 2).
@@ -1396,7 +1456,7 @@ struct Engine {
     if (dyn > 0) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(c.team_ctas);
-    lc.blockDim = dim3(c.block);
+    lc.blockDim = dim3(cta_threads(N, sc, c));
     lc.dynamicSmemBytes = dyn;
     lc.stream = stream;
     cudaLaunchAttribute at[1];
@@ -1424,22 +1484,23 @@ struct Engine {
     if (!k)
       return fail(HEOM_EUNSUPPORTED, "no engine kernel for N=%d, launch mode %d, node_threads %d%s", N, c.mode, c.G,
                   no_kernel_reason(N, sc));
+    const int block = cta_threads(N, sc, c);
     if (c.mode == 1) {
       int per_sm = 0;
       if (dyn > 0) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
-      CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, c.block, dyn));
-      if (per_sm < 1) return fail(HEOM_ECUDA, "block of %d threads cannot be resident", c.block);
+      CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, dyn));
+      if (per_sm < 1) return fail(HEOM_ECUDA, "block of %d threads cannot be resident", block);
       const int grid = per_sm * sms;
       CUDA_TRY(cudaMemsetAsync(A.gsync, 0, sizeof(unsigned), stream));
       void* args[] = {&A, &B};
-      CUDA_TRY(cudaLaunchCooperativeKernel(k, dim3(grid), dim3(c.block), args, dyn, stream));
+      CUDA_TRY(cudaLaunchCooperativeKernel(k, dim3(grid), dim3(block), args, dyn, stream));
       return HEOM_OK;
     }
     if (c.team_ctas > 8) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     if (dyn > 0) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(nteams * c.team_ctas);
-    lc.blockDim = dim3(c.block);
+    lc.blockDim = dim3(block);
     lc.dynamicSmemBytes = dyn;
     lc.stream = stream;
     cudaLaunchAttribute at[1];
@@ -1888,7 +1949,7 @@ int heom_autotune(heom_ctx* ctx, int64_t trial_steps, double* best_us_per_step) 
   TRY(e.ensure_device());
   Instance& in = *e.inst[0];
   // snapshot the state
-  const size_t arr = (size_t)in.N * in.N * in.Mpad * e.rsize();
+  const size_t arr = heom::state_reals(in.N, in.Mpad) * e.rsize();
   DevBuf sy, sr, sa;
   TRY(sy.alloc(arr, e.hooks));
   TRY(sr.alloc(in.root64.bytes, e.hooks));
@@ -1926,7 +1987,7 @@ int heom_autotune(heom_ctx* ctx, int64_t trial_steps, double* best_us_per_step) 
       // are refused by the launch
       const int U = in.N * (in.N + 1) / 2;
       for (int npt = 1; npt <= heom::kFlowMaxNpt; ++npt) {
-        if (!heom::flow_kernel(e.prec == HEOM_FP64, in.complex_h != 0, in.N, npt)) continue;
+        if (!e.flow_kernel_shape(in.complex_h != 0, in.N, npt)) continue;
         const int maxthr = npt == 1 ? heom::kFlowMaxThreads : heom::kFlowMaxThreadsMulti;
         for (int S : {4, 6, 8, 9, 10, 12, 13, 16, 24, 32, 64}) {
           if (S * U > maxthr) continue;
@@ -1963,8 +2024,9 @@ int heom_autotune(heom_ctx* ctx, int64_t trial_steps, double* best_us_per_step) 
   for (const LaunchCfg& c : cands) {
     e.cfg[in.N] = c;
     const int dyn = large ? heom::large_smem_bytes(in.N, (int)e.rsize())
-                          : (c.mode == 2 ? heom::smem_dyn_bytes(in.N, Engine::smem_slice(in.M, c.team_ctas))
-                                         : heom::engine_dyn_bytes(in.N, c.block, (int)e.rsize(), c.G <= 2));
+                    : c.mode == 2 ? heom::smem_dyn_bytes(in.N, Engine::smem_slice(in.M, c.team_ctas))
+                    : Engine::block_engine(in.N, in.scaled, c) ? e.block_dyn(in.N, c, in.M)
+                                                               : 0;
     if (c.mode != 1 && c.mode != 3 && e.max_active_teams(in.N, in.complex_h, in.scaled, c, dyn) < 1) {
       t_err.clear();
       continue;
@@ -2168,7 +2230,7 @@ int heom_batch_autotune(heom_batch* b, int64_t trial_steps, double* best_ms) {
   std::vector<DevBuf> sy(count), sr(count), sa(count);
   for (int i = 0; i < count; ++i) {
     Instance& in = *e.inst[i];
-    const size_t arr = (size_t)in.N * in.N * in.Mpad * e.rsize();
+    const size_t arr = heom::state_reals(in.N, in.Mpad) * e.rsize();
     TRY(sy[i].alloc(arr, e.hooks));
     TRY(sr[i].alloc(in.root64.bytes, e.hooks));
     TRY(sa[i].alloc(in.acc.bytes, e.hooks));
@@ -2233,7 +2295,7 @@ int heom_batch_autotune(heom_batch* b, int64_t trial_steps, double* best_ms) {
   e.cfg = best;
   for (int i = 0; i < count; ++i) {
     Instance& in = *e.inst[i];
-    const size_t arr = (size_t)in.N * in.N * in.Mpad * e.rsize();
+    const size_t arr = heom::state_reals(in.N, in.Mpad) * e.rsize();
     CUDA_TRY(cudaMemcpyAsync(in.y.p, sy[i].p, arr, cudaMemcpyDeviceToDevice, e.stream));
     CUDA_TRY(cudaMemcpyAsync(in.root64.p, sr[i].p, in.root64.bytes, cudaMemcpyDeviceToDevice, e.stream));
     CUDA_TRY(cudaMemcpyAsync(in.acc.p, sa[i].p, in.acc.bytes, cudaMemcpyDeviceToDevice, e.stream));
@@ -2331,7 +2393,8 @@ extern "C" int heom_propagate_static(const heom_params* params, const double* d_
   const size_t o_dn = align256(o_up + tab_bytes);
   const size_t o_ngam = align256(o_dn + tab_bytes);
   const size_t ngam_bytes = (size_t)Mpad * rs;
-  const size_t arr = (size_t)N * N * Mpad * rs;
+  const size_t arr = heom::state_reals(N, Mpad) * rs;
+  const size_t live = (size_t)N * N * Mpad * rs;
   const size_t o_y = align256(o_ngam + ngam_bytes);
   const size_t o_wa = align256(o_y + arr);
   const size_t o_wb = align256(o_wa + arr);
@@ -2392,6 +2455,7 @@ extern "C" int heom_propagate_static(const heom_params* params, const double* d_
   d.K = p.K;
   d.M = (int32_t)M;
   d.Mpad = Mpad;
+  d.rstride = 32;
   d.complex_h = complex_h;
   d.terminator = p.terminator;
   d.up = reinterpret_cast<const int32_t*>(base + o_up);
@@ -2417,16 +2481,16 @@ extern "C" int heom_propagate_static(const heom_params* params, const double* d_
   const int32_t team[4] = {0, 1, 0, 0};  // team_first = {0, 1}, team_list = {0}
 
   // one team (a thread-block cluster) for the single hierarchy
-  const int block = 256;
-  const int G = N >= 4 ? 8 : 2;
-  const int64_t units = ((M + 31) / 32) * G;
-  int ctas = (int)std::min<int64_t>(16, std::max<int64_t>(1, (units + block / 32 - 1) / (block / 32)));
-  int p2 = 1;
-  while (p2 < ctas) p2 <<= 1;
-  ctas = std::min(16, p2);
-  const void* k = heom::engine_kernel(fp64, complex_h != 0, G <= 2, N);
+  const int block = fp64 ? 256 : 512;
+  const int G = 2;  // the throughput engine: about one block of 32 nodes per CTA while the cluster reaches
+  int ctas = 1;
+  while (ctas < 16 && (int64_t)ctas * 32 < M) ctas <<= 1;
+  const void* k = heom::engine_kernel(fp64, complex_h != 0, G, N);
   if (!k) return fail(HEOM_EUNSUPPORTED, "no engine kernel for N=%d", N);
-  const int dyn = heom::engine_dyn_bytes(N, block, fp64 ? 8 : 4, G <= 2);
+  const int sets = heom::block_sets(N, (int)rs, block);
+  const int threads = 32 * N * sets;
+  const int dyn = heom::block_exch_bytes(N, (int)rs, sets);
+  int link_cache = 0;
   if (dyn > 0) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
   cudaLaunchConfig_t lc = {};
   cudaLaunchAttribute at[1];
@@ -2434,7 +2498,7 @@ extern "C" int heom_propagate_static(const heom_params* params, const double* d_
     if (ctas > 8) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     lc = cudaLaunchConfig_t{};
     lc.gridDim = dim3(ctas);
-    lc.blockDim = dim3(block);
+    lc.blockDim = dim3(threads);
     lc.dynamicSmemBytes = dyn;
     lc.stream = stream;
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -2454,6 +2518,8 @@ extern "C" int heom_propagate_static(const heom_params* params, const double* d_
   // everything that must start at zero: status and barrier words, the state
   CUDA_TRY(cudaMemsetAsync(base + o_status, 0, o_acc - o_status, stream));
   CUDA_TRY(cudaMemsetAsync(base + o_y, 0, arr, stream));
+  CUDA_TRY(cudaMemsetAsync(base + o_wa + live, 0, arr - live, stream));
+  CUDA_TRY(cudaMemsetAsync(base + o_wb + live, 0, arr - live, stream));
   CUDA_TRY(cudaMemcpyAsync(base + o_coef, h_coef, coef_bytes, cudaMemcpyHostToDevice, stream));
   CUDA_TRY(cudaMemcpyAsync(base + o_up, h_up, tab_bytes, cudaMemcpyHostToDevice, stream));
   CUDA_TRY(cudaMemcpyAsync(base + o_dn, h_dn, tab_bytes, cudaMemcpyHostToDevice, stream));
@@ -2479,7 +2545,7 @@ extern "C" int heom_propagate_static(const heom_params* params, const double* d_
   A.team_ctas = ctas;
   A.gsync = reinterpret_cast<unsigned*>(base + o_gsync);
   A.status = reinterpret_cast<int*>(base + o_status);
-  void* args[] = {&A};
+  void* args[] = {&A, &link_cache};
   CUDA_TRY(cudaLaunchKernelExC(&lc, k, args));
   if (d_rho_out) {
     if (fp64)
@@ -2628,7 +2694,7 @@ size_t request_bytes(const heom_params& p, bool tables_cached) {
   const size_t NN = (size_t)p.N * p.N;
   size_t coef = rs == 8 ? CoefLayout<double>::bytes(p.N) : CoefLayout<float>::bytes(p.N);
   if (p.flags & HEOM_FLAG_SCALED) coef = (coef + 15) / 16 * 16 + rs * 2 * (size_t)(p.K + 2) * p.N;
-  size_t b = 3 * r(NN * Mpad * rs) + r(Mpad * rs) + r(3 * 8 * NN + 32 * heom::kPartBytes) + r(coef) +
+  size_t b = 3 * r(heom::state_reals(p.N, (int)Mpad) * rs) + r(Mpad * rs) + r(3 * 8 * NN + 32 * heom::kPartBytes) + r(coef) +
              r(kAccDoubles * 8) + r(2 * 8 * NN);
   if (!tables_cached) b += 2 * r(4 * (size_t)p.N * Mpad);
   return b;
@@ -2662,38 +2728,23 @@ struct heom_server {
     if (host_mem) cudaFreeHost(host_mem);
   }
 
-  // Team of a request: about 256 nodes per CTA (1..16 CTAs), the hierarchy in
-  // the team's shared memory when it fits.
+  // Team of a request: about 256 nodes per CTA (1..16 CTAs).
   static int team_for(int64_t M) {
     int c = 1;
     while (c < 16 && (int64_t)c * 256 < M) c <<= 1;
     return c;
   }
-  // Launch shape of a request.  Scaled hierarchies (N <= 8) take a load view
-  // in device memory.  (Smaller teams -- 2 CTAs, or the fewest whose shared
+  // Launch shape of a request: the throughput engine.  (Smaller teams -- 2 CTAs, or the fewest whose shared
   // memory holds the hierarchy -- were measured slower on the serving trace:
   // the largest requests' service time then sets the makespan.)
-  static LaunchCfg launch_for(int prec, int N, int64_t M, int max_dyn, bool scaled) {
+  static LaunchCfg launch_for(int prec, int N, int64_t M, bool scaled) {
     LaunchCfg c;
     c.mode = 0;
     c.team_ctas = team_for(M);
     c.block = prec == HEOM_FP64 ? 256 : 512;
-    c.G = 2;
-    if (scaled && N <= heom::kMaxSmallN) {
-      c.G = std::max(3, std::min(8, N * (N + 1) / 2));
-      return c;
-    }
-    if (prec == HEOM_FP32_MIXED && N <= heom::kMaxSmallN &&
-        heom::smem_dyn_bytes(N, Engine::smem_slice(M, c.team_ctas)) <= max_dyn)
-      c.mode = 2;
+    c.G = scaled ? 4 : 2;
     return c;
   }
-  int max_dyn_smem() const {
-    int optin = 0;
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
-    return optin - 4096;
-  }
-
   int start_launch(int li, const std::vector<int64_t>& ids) {
     Launch& L = launches[li];
     auto eng = std::make_unique<Engine>();
@@ -2811,7 +2862,6 @@ struct heom_server {
     }
     size_t budget = arena.in_use;
     std::set<std::pair<int, int>> new_tables;
-    const int max_dyn = max_dyn_smem();
     while (!queue.empty()) {
       Request& q = *reqs[queue.front()];
       const auto tkey = std::make_pair(q.p.N, q.p.K);
@@ -2820,7 +2870,7 @@ struct heom_server {
       if (budget + need > arena.bytes) break;
       const int64_t M = heom::num_nodes(q.p.N, q.p.K);
       const bool sc = (q.p.flags & HEOM_FLAG_SCALED) != 0;
-      const LaunchCfg c = launch_for(q.p.precision, q.p.N, M, max_dyn, sc);
+      const LaunchCfg c = launch_for(q.p.precision, q.p.N, M, sc);
       const auto gkey = std::make_tuple(q.p.precision, q.p.N, c.team_ctas, c.mode, (int)sc);
       if (!groups.count(gkey)) {
         if (groups.size() == free_streams.size()) {  // no stream for a new group
