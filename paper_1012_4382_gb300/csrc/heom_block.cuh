@@ -18,7 +18,7 @@
 //
 // All warps run the same code: sites are counted relative to the warp's own
 // (r = a - b mod N), with the couplings rotated accordingly in shared memory,
-// and the state is in cyclic order during a call (cyc_pair), so that every
+// and the state is in cyclic order during a call (see cyc_pair), so that every
 // element is at a compile-time offset from one of 2 + N/2 addresses and the two
 // reals of a pair are one load.  N bodies
 // with compile-time columns were 43 KB of code at N = 7 and waited on
@@ -63,39 +63,6 @@ __host__ __device__ constexpr int block_sets(int N, int rsize, int block) {
   return s < 1 ? 1 : (s < block_max_sets(N, rsize) ? s : block_max_sets(N, rsize));
 }
 
-// Cyclic order of a state array (during a call): per block of 32 nodes the
-// diagonals, [N][32], then the pairs, [N(N-1)/2][32][2] (real part of sigma_{b,
-// b+d}, imaginary part), pair (b, b+d mod N), d = 1..(N-1)/2, at (d-1)N + b; for
-// even N the N/2 pairs (b, b+N/2), b < N/2, come last.  Both reals of a pair are
-// one load.  Places below are in units of one lane's real (diagonals) or of
-// two (pairs), times 32.
-__host__ __device__ constexpr int cyc_pair(int N, int d) { return (d - 1) * N; }  // of pair (0, d)
-// Pair {r, c}, r != c: its place; *rev: stored as (c', r') with c' the larger site.
-__host__ __device__ constexpr int cyc_place(int N, int r, int c, bool* rev) {
-  const int lo = r < c ? r : c, hi = r < c ? c : r, d = hi - lo;
-  const bool fwd = 2 * d <= N;  // pair (lo, lo + d); else (hi, hi + (N - d))
-  *rev = !fwd;
-  return cyc_pair(N, fwd ? d : N - d) + (fwd ? lo : hi);
-}
-// Index of packed element (r, c) (r <= c: Re sigma_rc, r > c: Im sigma_cr) of
-// lane l within its block; *neg: stored with the opposite sign.
-__host__ __device__ constexpr int cyc_index(int N, int r, int c, int l, bool* neg) {
-  *neg = false;
-  if (r == c) return r * 32 + l;
-  bool rev = false;
-  const int k = cyc_place(N, r, c, &rev);
-  *neg = rev && r > c;
-  return N * 32 + (k * 32 + l) * 2 + (r > c ? 1 : 0);
-}
-// The same within the root's own arrays: diagonals, then the two reals of every pair.
-__host__ __device__ constexpr int root_index(int N, int r, int c, bool* neg) {
-  *neg = false;
-  if (r == c) return r;
-  bool rev = false;
-  const int k = cyc_place(N, r, c, &rev);
-  *neg = rev && r > c;
-  return N + 2 * k + (r > c ? 1 : 0);
-}
 template <typename R>
 struct Vec2;
 template <>
@@ -517,7 +484,7 @@ __global__ void __launch_bounds__(block_max_threads(N, (int)sizeof(R)), 1) heom_
         if (s_rows.os.now) s_rows.rows.pending = s_rows.os.row++;
         s_rows.os.now = t + 2 == I.out_every * s_rows.os.row;
       }
-      if (I.stop_trace > 0.0 && t + 1 < I.nsteps && stop_now<R, MIXED>(I, N, &s_stop, 1)) {
+      if (I.stop_trace > 0.0 && t + 1 < I.nsteps && stop_now<R, MIXED>(I, N, &s_stop, 32)) {
         if (owner) s_rows.ea[col].store(I, col);
         done = t + 1;
         if (!team_barrier(A, epoch)) return;

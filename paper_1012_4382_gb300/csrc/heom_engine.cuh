@@ -60,7 +60,7 @@ struct Inst {
   int32_t N, K, M, Mpad;
   int32_t complex_h, terminator;
   int32_t wstride;     // scaled hierarchy: K + 2, the row length of wsc
-  int32_t rstride;     // stride between the root's elements in a state array: 32 (N <= 8), Mpad (N > 8)
+  int32_t dstride;     // distance between the root's diagonal elements in a state array
   const int32_t* up;   // [N][Mpad] index of n + e_j or -1
   const int32_t* dn;   // [N][Mpad] (n_j << 24) | index of n - e_j, or -1
   void* y;             // packed state (R), see state_elem; N <= 8: ended by a block of zeros
@@ -144,21 +144,68 @@ __device__ __forceinline__ void static_for(F&& f) {
   }
 }
 
-// Layout of a state array.  N <= 8: blocks of 32 nodes, [Mpad/32][N*N][32] --
-// element p of node n at node_col<N>(n) + 32 p, so that every element of a
-// node (and of a neighbour) is at a compile-time offset from one address --
-// followed by one more block that stays zero, which absent neighbours read.
-// N > 8: element-major, [N*N][Mpad].
+// Layout of a state array: blocks of 32 nodes, N*N*32 reals each, followed by
+// one more block that stays zero, which absent neighbours read.  Within a block,
+// N <= 8: packed element p of node n at node_col<N>(n) + 32 p, so that every
+// element of a node (and of a neighbour) is at a compile-time offset from one
+// address.  N > 8: cyclic order (cyc_index; heom_large.cuh keeps it between calls).
 template <int N>
 __host__ __device__ __forceinline__ constexpr unsigned node_col(int n) {
   return (unsigned)(n >> 5) * (N * N * 32) + (n & 31);
 }
-__host__ __device__ __forceinline__ size_t state_elem(int N, int Mpad, int p, int64_t n) {
-  return N <= kMaxSmallN ? ((size_t)(n >> 5) * (N * N) + p) * 32 + (n & 31) : (size_t)p * Mpad + n;
+// Cyclic order: per block the diagonals, [N][32], then the pairs,
+// [N(N-1)/2][32][2] (real part of sigma_{b,b+d}, imaginary part), pair (b, b+d mod N),
+// d = 1..(N-1)/2, at (d-1)N + b; for even N the N/2 pairs (b, b+N/2), b < N/2,
+// come last.  Column b of a node then is at few addresses for every b, and both
+// reals of a pair are one load.
+__host__ __device__ constexpr int cyc_pair(int N, int d) { return (d - 1) * N; }  // place of pair (0, d)
+// Place of pair {r, c}, r != c; *rev: stored as (c', r') with c' the larger site.
+__host__ __device__ constexpr int cyc_place(int N, int r, int c, bool* rev) {
+  const int lo = r < c ? r : c, hi = r < c ? c : r, d = hi - lo;
+  const bool fwd = 2 * d <= N;  // pair (lo, lo + d); else (hi, hi + (N - d))
+  *rev = !fwd;
+  return cyc_pair(N, fwd ? d : N - d) + (fwd ? lo : hi);
 }
-__host__ __device__ __forceinline__ size_t state_reals(int N, int Mpad) {
-  return (size_t)N * N * (N <= kMaxSmallN ? Mpad + 32 : Mpad);
+// Index of packed element (r, c) (r <= c: Re sigma_rc, r > c: Im sigma_cr) of
+// lane l within its block; *neg: stored with the opposite sign.
+__host__ __device__ constexpr int cyc_index(int N, int r, int c, int l, bool* neg) {
+  *neg = false;
+  if (r == c) return r * 32 + l;
+  bool rev = false;
+  const int k = cyc_place(N, r, c, &rev);
+  *neg = rev && r > c;
+  return N * 32 + (k * 32 + l) * 2 + (r > c ? 1 : 0);
 }
+// The same within the root's own arrays: diagonals, then the two reals of every pair.
+__host__ __device__ constexpr int root_index(int N, int r, int c, bool* neg) {
+  *neg = false;
+  if (r == c) return r;
+  bool rev = false;
+  const int k = cyc_place(N, r, c, &rev);
+  *neg = rev && r > c;
+  return N + 2 * k + (r > c ? 1 : 0);
+}
+// Index of packed element p = r * N + c of node n in a state array; *neg as above.
+__host__ __device__ __forceinline__ size_t state_elem(int N, int p, int64_t n, bool* neg) {
+  *neg = false;
+  const size_t block = (size_t)(n >> 5) * (N * N * 32);
+  return block + (N <= kMaxSmallN ? p * 32 + (int)(n & 31) : cyc_index(N, p / N, p % N, (int)(n & 31), neg));
+}
+template <typename R>
+__device__ __forceinline__ double state_get(const R* y, int N, int p, int64_t n) {
+  bool neg;
+  const double v = (double)y[state_elem(N, p, n, &neg)];
+  return neg ? -v : v;
+}
+template <typename R>
+__device__ __forceinline__ void state_put(R* y, int N, int p, int64_t n, double v) {
+  bool neg;
+  const size_t i = state_elem(N, p, n, &neg);
+  y[i] = (R)(neg ? -v : v);
+}
+__host__ __device__ __forceinline__ size_t state_reals(int N, int Mpad) { return (size_t)N * N * (Mpad + 32); }
+// Distance between a node's diagonal elements.
+__host__ __device__ constexpr int diag_stride(int N) { return N <= kMaxSmallN ? (N + 1) * 32 : 32; }
 
 // pair index u -> (a, b), a < b, in the order (0,1),(0,2),...,(1,2),...
 __host__ __device__ constexpr int pair_a(int N, int u) {
@@ -1103,7 +1150,7 @@ __device__ __forceinline__ void write_row0(const Inst& I) {
   if (I.out_pops)
     for (int a = 0; a < N; ++a)
       I.out_pops[a] = MIXED ? ff_to_double(static_cast<const FF*>(I.y0)[a * N + a])
-                            : (double)static_cast<const R*>(I.y)[(a * N + a) * I.rstride];
+                            : (double)static_cast<const R*>(I.y)[a * I.dstride];
   if (I.out_el) {
     I.out_el[0] = I.acc[0];
     I.out_el[1] = I.acc[1];
@@ -1169,9 +1216,9 @@ struct EtaRows {
 // The stop rule: true when the site population of the root after the step
 // just finished is below I.stop_trace.  Every CTA of the team evaluates it
 // from the same memory after the stage barrier, so all take the same branch.
-// dstep: distance of the root's diagonal elements in y's order (0: packed order, N + 1).
+// dstride: distance of the root's diagonal elements in y (0: I.dstride).
 template <typename R, bool MIXED>
-__device__ __forceinline__ bool stop_now(const Inst& I, int N, int* s_flag, int dstep = 0) {
+__device__ __forceinline__ bool stop_now(const Inst& I, int N, int* s_flag, int dstride = 0) {
   if (threadIdx.x == 0) {
     double tr = 0.0;
     if constexpr (MIXED) {
@@ -1181,8 +1228,8 @@ __device__ __forceinline__ bool stop_now(const Inst& I, int N, int* s_flag, int 
       tr = ff_to_double(sum);
     } else {
       const R* y = static_cast<const R*>(I.y);
-      if (dstep == 0) dstep = N + 1;
-      for (int a = 0; a < N; ++a) tr += (double)__ldcg(y + (size_t)(a * dstep) * I.rstride);
+      if (dstride == 0) dstride = I.dstride;
+      for (int a = 0; a < N; ++a) tr += (double)__ldcg(y + a * dstride);
     }
     *s_flag = tr < I.stop_trace;
   }
@@ -1204,7 +1251,7 @@ __device__ __forceinline__ void finish_instance(const Inst& I, int nslots, const
       const float* y0 = static_cast<const float*>(I.y0);
       flag_nonfinite(status, (double)__ldcg(y0 + 2 * (a * N + a)) + (double)__ldcg(y0 + 2 * (a * N + a) + 1));
     } else {
-      flag_nonfinite(status, (double)__ldcg(static_cast<const R*>(I.y) + (size_t)(a * N + a) * I.rstride));
+      flag_nonfinite(status, (double)__ldcg(static_cast<const R*>(I.y) + a * I.dstride));
     }
   }
   if (done < I.nsteps) {

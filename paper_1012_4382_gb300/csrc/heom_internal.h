@@ -19,8 +19,15 @@ const void* block_kernel_f32_cplx(int N);
 // Scaled hierarchies (HEOM_FLAG_SCALED), N = 1..8, load views.
 const void* engine_kernel_scaled_f64(int N, bool cplx);
 const void* engine_kernel_scaled_f32(int N, bool cplx);
-// Large-N engine (9..24 sites).
-const void* large_kernel(bool fp64, bool cplx, bool scaled);
+// Large-N engine for N = 9..24 (nullptr otherwise), scaled hierarchies included.
+const void* large_kernel_f64_real(int N);
+const void* large_kernel_f64_cplx(int N);
+const void* large_kernel_f32_real(int N);
+const void* large_kernel_f32_cplx(int N);
+inline const void* large_kernel(bool fp64, bool cplx, int N) {
+  if (fp64) return cplx ? large_kernel_f64_cplx(N) : large_kernel_f64_real(N);
+  return cplx ? large_kernel_f32_cplx(N) : large_kernel_f32_real(N);
+}
 // Dataflow engine (launch mode 3, one hierarchy on the whole GPU), N = 1..8,
 // npt nodes per thread (nullptr where that count is not built).
 const void* flow_kernel_f32(int N, bool cplx, int npt);

@@ -1,39 +1,355 @@
-// Large-N engine of the HEOM RK4 propagation (9..24 sites): see the comment
-// below.  Shares the descriptors, coefficient layout, barriers, eta sums and
-// stop rule of heom_engine.cuh.
+// heom_large.cuh -- the engine for hierarchies with 9..24 sites.  Shares the
+// descriptors, coefficient layout, barriers, eta sums and stop rule of
+// heom_engine.cuh and the column form and cyclic order of heom_block.cuh:
+//
+//   D = P + P^+ + (local terms),  P = -i Q, column b of Q from column b of the
+//   node and the links of site b:
+//   Q_ab = (H' sigma)_ab + w_b sigma_{n+e_b, ab} + n_b (alpha_b + i beta_b) sigma_{n-e_b, ab}
+//
+// 32 consecutive nodes (one lane each) are computed by a set of warps of one
+// CTA, a warp taking whole columns.  The state stays in cyclic order (state_elem),
+// where pair (b, b+d) belongs to column b.  A block is done in two phases: the
+// lower half of every column (its pairs (b-d, b), which their other column
+// finishes) goes to the exchange area in shared memory; after a barrier the
+// upper half (the diagonal and the pairs (b, b+d)) is computed, completed with
+// the exchanged elements and the local terms, and stored.  So a thread holds
+// the accumulators of half a column (26 registers in FP32, 52 in FP64 at N =
+// 24), and every coupling read from shared memory (a broadcast) serves two
+// multiply-adds, in FP32 one packed instruction.
+//
+// FP32 first brings the block's stage input (74 KB at N = 24) into shared
+// memory, since the two phases and the two columns of a pair read every element
+// four times; FP64, bound by its pipe, reads it through L1.  Links that no lane
+// of the warp has (most: a node of depth 4 has at most four nonzero n_j) are
+// skipped by a vote, with their arithmetic.
 #pragma once
 
-#include "heom_engine.cuh"
+#include "heom_block.cuh"
 
 namespace heom {
 
-// ------------------------------------------------------------ large-N engine
-//
-// Hierarchies with 9..24 sites (N is a run-time argument).  A CTA stages a
-// tile of 16 consecutive nodes' matrices in shared memory, element-major with
-// the 16 nodes innermost; two lanes share a node (lane = 2 x node + half), so
-// a warp covers the 16 nodes and every shared-memory access is free of bank
-// conflicts (the two lanes of a node read the same word).  The node's outputs
-// are cut into 4 x 4 blocks (a in A, b in B, A <= B, the upper triangle);
-// warp w computes blocks w, w + nwarps, ... of all 16 nodes, each lane two
-// rows of a block.  Within a block the commutator is a small matrix product:
-// for each k the thread reads sigma_ak for its two rows and sigma_kb for the
-// four columns, row k of J, and does 32 multiply-adds.  Neighbours are read
-// from device memory.  Teams and barriers are those of the small-N engine.
-//
-// FP32 keeps Re sigma and Im sigma in the tile as full, zero-padded
-// 4 ceil(N/4)-square matrices (no selects in the product loop); FP64 keeps
-// the packed matrix.  The 16-node tile (74 KB at N = 24) lets two FP32 CTAs share
-// an SM, so one CTA's loads overlap the other's arithmetic.
-constexpr int kLargeTile = 16;
+// Columns a warp takes, sets of a CTA, warps of a set.  FP32: a warp per column
+// and 18 to 24 warps; FP64: two columns a warp (168 or 128 registers a thread).
+__host__ __device__ constexpr int large_cols(int rsize) { return rsize == 8 ? 2 : 1; }
+__host__ __device__ constexpr int large_set_warps(int N, int rsize) { return (N + large_cols(rsize) - 1) / large_cols(rsize); }
+__host__ __device__ constexpr int large_sets(int N, int rsize) { return N <= (rsize == 8 ? 16 : 12) ? 2 : 1; }
+__host__ __device__ constexpr int large_threads(int N, int rsize) {
+  return 32 * large_set_warps(N, rsize) * large_sets(N, rsize);
+}
+// Coupling table: two copies (the second shifted by one entry, so that a row's
+// part can be read two entries at a time from any column) of [N][2N] entries of
+// 8 bytes: a double, or a float twice.
+__host__ __device__ constexpr int large_jrow(int N) { return 2 * N + 4; }
+__host__ __device__ constexpr int large_jbytes(int N) { return 2 * N * large_jrow(N) * 8; }
+__host__ __device__ constexpr int large_stage_bytes(int N, int rsize) { return rsize == 4 ? N * N * 32 * 4 : 0; }
+__host__ __device__ constexpr int large_exch_bytes(int N, int rsize) { return N * (N - 1) * 32 * rsize; }
+__host__ __device__ constexpr int large_smem_bytes(int N, int rsize, bool cplx) {
+  return (cplx ? 2 : 1) * large_jbytes(N) +
+         large_sets(N, rsize) * (large_stage_bytes(N, rsize) + large_exch_bytes(N, rsize));
+}
 
-// SC: scaled hierarchy, link weights from Inst::wsc (see scaled_up).
-template <typename R, bool MIXED, bool CPLX, bool SC = false>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) heom_large_kernel(EngineArgs A) {
+// A coupling entry and its multiply-add on a complex accumulator.
+template <typename R>
+struct Coupling;
+template <>
+struct Coupling<double> {
+  typedef double type;
+  static __device__ __forceinline__ double make(double v) { return v; }
+  static __device__ __forceinline__ void fma2(double2& acc, double j, double2 v) {
+    acc.x = fma(j, v.x, acc.x);
+    acc.y = fma(j, v.y, acc.y);
+  }
+};
+template <>
+struct Coupling<float> {
+  typedef float2 type;
+  static __device__ __forceinline__ float2 make(float v) { return make_float2(v, v); }
+  static __device__ __forceinline__ void fma2(float2& acc, float2 j, float2 v) {
+    asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%0, %1};\n\t"
+        "fma.rn.f32x2 c, a, b, c;\n\tmov.b64 {%0, %1}, c;\n\t}"
+        : "+f"(acc.x), "+f"(acc.y)
+        : "f"(j.x), "f"(j.y), "f"(v.x), "f"(v.y));
+  }
+};
+template <typename R>
+struct alignas(16) CouplingPair {
+  typename Coupling<R>::type a, b;
+};
+
+// Barrier of `threads` threads; true when `fail` is set on any of them.
+__device__ __forceinline__ void set_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void copy16_async(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+template <int N, typename R>
+struct LargeCoef {
+  alignas(16) R site[2 * N][4];  // eps, goff, alpha, beta of site a at [a] and [a + N]
+  R gam[N], gd[N];
+};
+
+// What the columns of one item share.
+template <typename R>
+struct LargeItem {
+  StageArgs<R> S;
+  const R* win;    // the block's stage input: in shared memory (FP32) or device memory
+  int nb, lane;
+  R ng;
+};
+
+// Half of column b of Q: rows r0..r0+NR-1 (sites b + r).  BACK: the pairs (b-d, b), r = N-D..N-1; else the diagonal
+// and the pairs (b, b+d), r = 0..D.  HALF (even N): with the pair at distance N/2.
+template <int N, typename R, bool CPLX, bool BACK, bool HALF>
+struct HalfColumn {
+  typedef typename Vec2<R>::type R2;
+  typedef typename Coupling<R>::type JT;
+  static constexpr int D = (N - 1) / 2;
+  static constexpr int NR = (BACK ? D : D + 1) + (HALF ? 1 : 0);
+  static constexpr int r0 = BACK ? (HALF ? N / 2 : N - D) : 0;
+  R2 acc[NR];
+
+  // place of the pair {b, b + r} (times 32), and whether its stored imaginary part is that of sigma_{b, b+r}
+  static __device__ __forceinline__ int place(int r, int b) {
+    if (2 * r < N) return (r - 1) * N + b;
+    if (2 * r == N) return (N / 2 - 1) * N + (2 * b < N ? b : b - N / 2);
+    const int d = N - r;
+    return (d - 1) * N + (b >= d ? b - d : b - d + N);
+  }
+  static __device__ __forceinline__ bool forward(int r, int b) { return 2 * r < N || (2 * r == N && 2 * b < N); }
+
+  // acc += J(b + k, b + r) v over the rows r
+  __device__ __forceinline__ void couple(const JT* jt, const JT* jti, int b, int site_k, R2 v) {
+    const int c0 = b + r0, copy = c0 & 1;
+    const JT* row = jt + (copy * N + site_k) * large_jrow(N) + c0 + copy;
+    static_for<0, (NR + 1) / 2>([&](auto ic) {
+      constexpr int i = 2 * decltype(ic)::value;
+      const CouplingPair<R> j = *reinterpret_cast<const CouplingPair<R>*>(row + i);
+      Coupling<R>::fma2(acc[i], j.a, v);
+      if constexpr (i + 1 < NR) Coupling<R>::fma2(acc[i + 1], j.b, v);
+    });
+    if constexpr (CPLX) {
+      const JT* ri = jti + (copy * N + site_k) * large_jrow(N) + c0 + copy;
+      const R2 w{-v.y, v.x};
+      static_for<0, (NR + 1) / 2>([&](auto ic) {
+        constexpr int i = 2 * decltype(ic)::value;
+        const CouplingPair<R> j = *reinterpret_cast<const CouplingPair<R>*>(ri + i);
+        // the table holds Ji(b + k, b + r) = -Ji(b + r, b + k); stored with that sign turned
+        Coupling<R>::fma2(acc[i], j.a, w);
+        if constexpr (i + 1 < NR) Coupling<R>::fma2(acc[i + 1], j.b, w);
+      });
+    }
+  }
+
+  __device__ __forceinline__ void compute(const LargeItem<R>& it, const LargeCoef<N, R>& cf, const JT* jt, const JT* jti,
+                                          int b, int up, int dn) {
+    const StageArgs<R>& S = it.S;
+#pragma unroll
+    for (int i = 0; i < NR; ++i) acc[i] = R2{R(0), R(0)};
+    const R* diag = it.win + it.lane;
+    const R2* pairs = reinterpret_cast<const R2*>(it.win + N * 32) + it.lane;
+    // H' sigma, column entry by column entry
+    couple(jt, jti, b, b, R2{diag[b * 32], R(0)});
+    {
+      const R2* p = pairs + b * 32;
+      int site = b;
+#pragma unroll 4
+      for (int k = 1; k <= D; ++k, p += N * 32) {
+        site = site + 1 == N ? 0 : site + 1;
+        const R2 v = *p;
+        couple(jt, jti, b, site, R2{v.x, -v.y});
+      }
+    }
+    if constexpr (N % 2 == 0) {
+      const bool low = 2 * b < N;
+      const R2 v = pairs[((N / 2 - 1) * N + (low ? b : b - N / 2)) * 32];
+      couple(jt, jti, b, low ? b + N / 2 : b - N / 2, R2{v.x, low ? -v.y : v.y});
+    }
+    {
+      int site = b;
+      const R2* p = pairs;
+#pragma unroll 4
+      for (int d = 1; d <= D; ++d, p += N * 32) {
+        site = site == 0 ? N - 1 : site - 1;
+        couple(jt, jti, b, site, p[site * 32]);
+      }
+    }
+    // links of site b
+    const R* sb = cf.site[b];
+    R w_dn = R((dn >> 24) & 0xFF), w_up = R(1);
+    if (S.wsc) {
+      const R n_b = dn < 0 ? R(0) : w_dn;
+      w_up = scaled_up(S.wsc, S.wstride, b, n_b);
+      w_dn = scaled_dn(S.wsc, S.wstride, b, n_b);
+    }
+    auto linked = [&](int l) { return S.win + (size_t)(l >= 0 ? (unsigned)(l >> 5) * (N * N * 32) : S.zero); };
+    if (__any_sync(0xFFFFFFFFu, dn >= 0)) {
+      const int m = dn < 0 ? -1 : (dn & 0xFFFFFF);
+      const R* g0 = linked(m) + (m & 31);
+      const R2* g = reinterpret_cast<const R2*>(linked(m) + N * 32) + (m & 31);
+      const R al = w_dn * sb[2], be = w_dn * sb[3];
+      static_for<0, NR>([&](auto ic) {
+        constexpr int i = decltype(ic)::value, r = r0 + i;
+        if constexpr (r == 0) {
+          acc[i].y += be * g0[b * 32];
+        } else {
+          const R2 v = g[place(r, b) * 32];
+          const R vi = forward(r, b) ? -v.y : v.y;
+          acc[i].x += al * v.x;
+          acc[i].x -= be * vi;
+          acc[i].y += al * vi;
+          acc[i].y += be * v.x;
+        }
+      });
+    }
+    if (__any_sync(0xFFFFFFFFu, up >= 0)) {
+      const R2* g = reinterpret_cast<const R2*>(linked(up) + N * 32) + (up & 31);
+      static_for<0, NR>([&](auto ic) {
+        constexpr int i = decltype(ic)::value, r = r0 + i;
+        if constexpr (r != 0) {
+          const R2 v = g[place(r, b) * 32];
+          acc[i].x += w_up * v.x;
+          if (forward(r, b)) acc[i].y -= w_up * v.y;
+          else acc[i].y += w_up * v.y;
+        }
+      });
+    }
+    // Markov terminator of a leaf node (see heom_block.cuh)
+    if (S.terminator) {
+      const R nj = dn < 0 ? R(0) : R(dn >> 24);
+      const R c = up < 0 ? (nj + R(1)) / (it.ng + cf.gam[b]) : R(0);
+      const R ca = c * sb[2], cb = c * sb[3];
+      static_for<0, NR>([&](auto ic) {
+        constexpr int i = decltype(ic)::value, r = r0 + i;
+        if constexpr (r != 0) {
+          const R2 v = pairs[place(r, b) * 32];
+          const R vi = forward(r, b) ? -v.y : v.y;
+          acc[i].x += cb * v.x;
+          acc[i].x += ca * vi;
+          acc[i].y += cb * vi;
+          acc[i].y -= ca * v.x;
+        }
+      });
+    }
+  }
+};
+
+// First phase: the elements of column b that other columns finish.
+template <int N, typename R, bool CPLX, bool HALF>
+__device__ __forceinline__ void large_hand_over(const LargeItem<R>& it, const LargeCoef<N, R>& cf,
+                                                const typename Coupling<R>::type* jt,
+                                                const typename Coupling<R>::type* jti, int b, int up, int dn,
+                                                typename Vec2<R>::type* ex) {
+  typedef HalfColumn<N, R, CPLX, true, HALF> C;
+  C c;
+  c.compute(it, cf, jt, jti, b, up, dn);
+  static_for<0, C::NR>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    ex[C::place(C::r0 + i, b) * 32] = typename Vec2<R>::type{c.acc[i].y, -c.acc[i].x};  // P = -i Q
+  });
+}
+
+// Second phase: the diagonal b and the pairs (b, b+d), the Horner update and the stores.
+template <int N, typename R, bool MIXED, bool CPLX, bool HALF>
+__device__ __forceinline__ void large_finish(const Inst& I, const LargeItem<R>& it, const LargeCoef<N, R>& cf,
+                                             const typename Coupling<R>::type* jt,
+                                             const typename Coupling<R>::type* jti, const double* __restrict__ cfd,
+                                             int b, int up, int dn, const typename Vec2<R>::type* ex,
+                                             BlockRows<N, R>& rw, BlockRoot<MIXED ? N : 1>& br) {
+  typedef typename Vec2<R>::type R2;
+  typedef HalfColumn<N, R, CPLX, false, HALF> C;
+  const StageArgs<R>& S = it.S;
+  const int lane = it.lane;
+  const size_t self = (size_t)it.nb * (N * N * 32);
+  C c;
+  c.compute(it, cf, jt, jti, b, up, dn);
+  const R* sb = cf.site[b];
+  const bool root = MIXED && it.nb == 0 && lane == 0;
+  const R* yd = S.yv + self;
+  const R2* yp = reinterpret_cast<const R2*>(yd + N * 32) + lane;
+  R* wd = S.wout + self + b * 32 + lane;
+  R2* wp = reinterpret_cast<R2*>(S.wout + self + N * 32) + lane;
+  const R2* pairs = reinterpret_cast<const R2*>(it.win + N * 32) + lane;
+  const R s0 = it.win[b * 32 + lane];
+  {
+    R d = R(2) * c.acc[0].y;
+    d -= (it.ng + R(2) * cf.gd[b]) * s0;
+    if (root) br.acc[b] = (float)d;
+    *wd = yd[b * 32 + lane] + S.h * d;
+  }
+  static_for<1, C::NR>([&](auto ic) {
+    constexpr int r = decltype(ic)::value;
+    const int k = (r - 1) * N + b;
+    const R2 o = ex[k * 32], v = pairs[k * 32], y = yp[k * 32];
+    const R* sa = cf.site[b + r];
+    const R w = sa[0] - sb[0], g = it.ng + (sa[1] + sb[1]);
+    R re = c.acc[r].y + o.x;
+    R im = o.y + c.acc[r].x;  // of sigma_{b, b+r}
+    re -= w * v.y;
+    re -= g * v.x;
+    im += w * v.x;
+    im -= g * v.y;
+    if (root) {
+      br.acc[N + 2 * k] = (float)re;
+      br.acc[N + 2 * k + 1] = (float)im;
+    }
+    wp[k * 32] = R2{y.x + S.h * re, y.y + S.h * im};
+  });
+  if (it.nb == 0) {
+    __syncwarp();
+    if constexpr (MIXED) {
+      // float-float update of the root's elements (lane 0 the diagonal, lanes 2d-1 and 2d the pair at distance d),
+      // their hi parts to column 0 for the neighbours
+      const int d = (lane + 1) / 2;
+      if (lane <= 2 * (C::NR - 1)) {
+        const int p = lane == 0 ? b : N + 2 * ((d - 1) * N + b) + ((lane + 1) & 1);
+        const FF w = ff_axpy(br.w[0][p], (float)S.h, S.hl, br.acc[p]);
+        if (lane == 0) {
+          if (S.s == 2) {
+            rw.ea[b].add_xi(I, b, br.w[S.in_sel][p]);
+            rw.ea[b].step_xi(I);
+          }
+          if (S.s == 3) {
+            rw.ea[b].add(I, b, br.w[S.in_sel][p]);
+            static_cast<FF*>(I.y0)[b * (N + 1)] = w;  // for the stop rule
+            if (rw.os.now && I.out_pops) I.out_pops[rw.os.row * N + b] = ff_to_double(w);
+          }
+        }
+        br.w[S.out_sel][p] = w;
+        S.wout[lane == 0 ? b * 32 : N * 32 + 64 * ((d - 1) * N + b) + ((lane + 1) & 1)] = w.h;
+      }
+    } else {
+      if (lane == 0) {
+        if (S.s == 2) {
+          rw.ea[b].add_xi(I, cfd, b, (double)s0);
+          rw.ea[b].step_xi(I);
+        }
+        if (S.s == 3) {
+          rw.ea[b].add(I, cfd, N, b, (double)s0);
+          if (rw.os.now && I.out_pops) I.out_pops[rw.os.row * N + b] = (double)*wd;
+        }
+      }
+    }
+  }
+}
+
+template <int N, typename R, bool MIXED, bool CPLX>
+__global__ void __launch_bounds__(large_threads(N, (int)sizeof(R)), 1) heom_large_kernel(EngineArgs A) {
   extern __shared__ __align__(16) unsigned char dsm[];
+  __shared__ LargeCoef<N, R> s_cf;
+  __shared__ double s_rates[2 * N];
+  __shared__ BlockRoot<MIXED ? N : 1> s_root;
+  __shared__ BlockRows<N, R> s_rows;
   __shared__ Inst s_inst;
   __shared__ int s_stop;
-  constexpr int TN = kLargeTile;
+  typedef typename Coupling<R>::type JT;
+  typedef typename Vec2<R>::type R2;
+  constexpr int NN = N * N;
+  constexpr int RS = (int)sizeof(R);
+  constexpr int SW = large_set_warps(N, RS), SETS = large_sets(N, RS);
+  constexpr bool STAGED = RS == 4, EVEN = N % 2 == 0;
 
   int team, rank, team_size;
   if (A.mode == 0) {
@@ -45,14 +361,15 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) heom_large_kernel
     rank = blockIdx.x;
     team_size = gridDim.x;
   }
-  const int nwarps = blockDim.x >> 5;
-  const int warp = threadIdx.x >> 5;
-  const int lane = threadIdx.x & 31;
-  const int node = lane >> 1, half = lane & 1;
-  // tile 0 is on rank 0; its node 0 is the root, on lanes 0 and 1 of every warp
-  const int nslots = 2 * nwarps;
-  const int slot = (rank == 0 && lane < 2) ? 2 * warp + lane : -1;
-  const bool lead = (rank == 0 && threadIdx.x == 0);
+  const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int set = wid / SW, sw = wid - set * SW;
+  const bool lead = rank == 0 && threadIdx.x == 0;
+  JT* const jt = reinterpret_cast<JT*>(dsm);
+  JT* const jti = reinterpret_cast<JT*>(dsm + (CPLX ? large_jbytes(N) : 0));
+  unsigned char* const area = dsm + (CPLX ? 2 : 1) * large_jbytes(N) +
+                              (size_t)set * (large_stage_bytes(N, RS) + large_exch_bytes(N, RS));
+  R* const stage = reinterpret_cast<R*>(area);
+  R2* const ex = reinterpret_cast<R2*>(area + large_stage_bytes(N, RS)) + lane;
   unsigned epoch = 0;
 
   for (int li = A.team_first[team]; li < A.team_first[team + 1]; ++li) {
@@ -60,430 +377,143 @@ __global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) heom_large_kernel
     if (threadIdx.x == 0) s_inst = A.insts[A.team_list[li]];
     __syncthreads();
     const Inst& I = s_inst;
-    const int N = I.N;
-    const int NN = N * N;
-    using L = CoefLayout<R>;
-    const int JS = L::JS(N);  // = 4 * number of blocks per side
-    const int NB = JS / 4;
-    const int nblk = NB * (NB + 1) / 2;
-    constexpr bool FULL = sizeof(R) == 4;
-    R* tile = reinterpret_cast<R*>(dsm);
-    R* tileA = tile + JS * JS * TN;
-    unsigned char* cbytes = dsm + (size_t)(FULL ? 2 * JS * JS : NN) * TN * sizeof(R);
-    const int cb = L::bytes(N);
-    for (int i = threadIdx.x; i < cb; i += blockDim.x) cbytes[i] = static_cast<const unsigned char*>(I.coef)[i];
-    if (FULL)
-      for (int i = threadIdx.x; i < 2 * JS * JS * TN; i += blockDim.x) tile[i] = R(0);  // padding stays 0
-    __syncthreads();
-    const R* cf = reinterpret_cast<const R*>(cbytes);
-    const double* cfd = reinterpret_cast<const double*>(cbytes + L::dbl_offset(N));
-    const R* ngam = static_cast<const R*>(I.ngam);
-    const int Mp = I.Mpad;
-    const int ntiles = (I.M + TN - 1) / TN;
-    EtaAcc<R> ea;
-    EtaRows rows;
-    rows.acc0 = I.acc[0];
-    rows.acc1 = I.acc[1];
-    if (lead) {
-      if (I.out_pops)
-        for (int a = 0; a < N; ++a)
-          I.out_pops[a] = MIXED ? ff_to_double(static_cast<const FF*>(I.y0)[a * N + a])
-                                : (double)static_cast<const R*>(I.y)[(a * N + a) * Mp];
-      if (I.out_el) {
-        I.out_el[0] = I.acc[0];
-        I.out_el[1] = I.acc[1];
+    {
+      using L = CoefLayout<R>;
+      const R* cf = static_cast<const R*>(I.coef);
+      const double* rates = reinterpret_cast<const double*>(static_cast<const unsigned char*>(I.coef) + L::dbl_offset(N));
+      constexpr int JR = large_jrow(N);
+      for (int i = threadIdx.x; i < 2 * N * JR; i += blockDim.x) {
+        const int copy = i / (N * JR), a = i / JR % N, c = i % JR - copy;
+        const int col = c < 0 ? 0 : c % N;  // entries outside 0..2N-1 are never used, only read
+        jt[i] = Coupling<R>::make(cf[L::J(N) + a * L::JS(N) + col]);
+        // Ji(b + r, b + k), read from row b + k
+        if constexpr (CPLX) jti[i] = Coupling<R>::make(-cf[L::Ji(N) + a * L::JS(N) + col]);
       }
-      for (int k = 0; k < nslots; ++k) ea.store(I, k);  // zero every running-sum slot of this instance
+      for (int i = threadIdx.x; i < 8 * N; i += blockDim.x) s_cf.site[i / 4][i % 4] = cf[L::site(N) + 4 * (i / 4 % N) + i % 4];
+      for (int i = threadIdx.x; i < N; i += blockDim.x) {
+        s_cf.gam[i] = cf[L::gam(N) + i];
+        s_cf.gd[i] = cf[L::gd(N) + i];
+        s_rates[i] = rates[i];
+        s_rates[N + i] = rates[N + i];
+      }
+    }
+    const int nblk = (I.M + 31) >> 5;
+    if (lead) {
+      s_rows.os = OutStep{I.out_every == 1, 1};
+      s_rows.rows.pending = -1;
+      s_rows.rows.acc0 = I.acc[0];
+      s_rows.rows.acc1 = I.acc[1];
+      write_row0<N, R, MIXED>(I);
+      for (int k = 0; k < N; ++k) {  // zero the running sums of every site
+        s_rows.ea[k] = EtaAcc<R>{};
+        s_rows.ea[k].store(I, k);
+      }
+    }
+    if constexpr (MIXED) {
+      for (int p = threadIdx.x; p < NN; p += blockDim.x) {
+        bool neg;
+        const int q = root_index(N, p / N, p % N, &neg);
+        const FF w = static_cast<const FF*>(I.y0)[p];
+        s_root.w[0][q] = neg ? FF{-w.h, -w.l} : w;
+      }
     }
     if (!team_barrier(A, epoch)) return;
-    R* arr[3] = {static_cast<R*>(I.y), static_cast<R*>(I.wa), static_cast<R*>(I.wb)};
-    int64_t next_out = I.out_every, orow = 1, done = I.nsteps;
+
+    int64_t done = I.nsteps;
     for (int64_t t = 0; t < I.nsteps; ++t) {
-      const OutStep os{t + 1 == next_out, orow};
-      if (os.now) {
-        next_out += I.out_every;
-        ++orow;
-      }
 #pragma unroll 1
       for (int s = 0; s < 4; ++s) {
-        if (s == 0 && rows.pending >= 0) {
-          if (lead) eta_write_row<R>(I, nslots, rows.acc0, rows.acc1, rows.pending, A.status);
-          rows.pending = -1;
+        if (s == 0 && lead && s_rows.rows.pending >= 0) {
+          eta_write_row<R>(I, N, s_rows.rows.acc0, s_rows.rows.acc1, s_rows.rows.pending, A.status);
+          s_rows.rows.pending = -1;
         }
         int in_sel, out_sel;
         stage_buffers(s, in_sel, out_sel);
-        const StageCoef<R> P = stage_coef<R>(I, s, in_sel, out_sel);
-        const R h = P.h;
-        const R* __restrict__ win = arr[in_sel];
-        R* __restrict__ wout = arr[out_sel];
-        const R* __restrict__ yv = arr[0];
-        for (int tl = rank; tl < ntiles; tl += team_size) {
-          const int n0 = tl * TN;
-          __syncthreads();
-          {
-            // thread t copies (element, node) pairs e = t, t + blockDim, ...,
-            // element e / 16 of node e % 16; 8 loads in flight before their
-            // stores; (r, c) of the packed element is stepped along.
-            const int jn = threadIdx.x & (TN - 1);
-            const bool lv = n0 + jn < I.M;
-            const int pstep = blockDim.x / TN;
-            int r0 = 0, c0 = threadIdx.x / TN;
-            while (c0 >= N) { c0 -= N; ++r0; }
-            for (int p0 = threadIdx.x / TN; p0 < NN; p0 += 8 * pstep) {
-              R v[8];
-              int rr[8], cc[8];
-              int r = r0, c = c0;
-#pragma unroll
-              for (int q = 0; q < 8; ++q) {
-                const int pp = p0 + q * pstep;
-                rr[q] = r;
-                cc[q] = c;
-                v[q] = ld_global_or0(win + (pp * Mp + n0 + jn), lv && pp < NN);
-                c += pstep;
-                while (c >= N) { c -= N; ++r; }
-              }
-              r0 = r;
-              c0 = c;
-#pragma unroll
-              for (int q = 0; q < 8; ++q) {
-                const int pp = p0 + q * pstep;
-                if (pp >= NN) break;
-                if constexpr (FULL) {
-                  // packed (r, c): Re sigma_rc for r <= c, Im sigma_cr for r > c
-                  const int rq = rr[q], cq = cc[q];
-                  if (rq < cq) {
-                    tile[(rq * JS + cq) * TN + jn] = v[q];
-                    tile[(cq * JS + rq) * TN + jn] = v[q];
-                  } else if (rq > cq) {
-                    tileA[(cq * JS + rq) * TN + jn] = v[q];
-                    tileA[(rq * JS + cq) * TN + jn] = -v[q];
-                  } else {
-                    tile[(rq * JS + rq) * TN + jn] = v[q];
-                  }
-                } else {
-                  tile[pp * TN + jn] = v[q];
-                }
-              }
+        LargeItem<R> it;
+        StageArgs<R>& S = it.S;
+        S.win = static_cast<const R*>(in_sel == 0 ? I.y : (in_sel == 1 ? I.wa : I.wb));
+        S.wout = static_cast<R*>(out_sel == 0 ? I.y : (out_sel == 1 ? I.wa : I.wb));
+        S.yv = static_cast<const R*>(I.y);
+        S.ngam = static_cast<const R*>(I.ngam);
+        S.zero = (unsigned)(I.Mpad >> 5) * (NN * 32);
+        S.h = RS == 8 ? (R)I.hd[s] : (R)I.hh[s];
+        S.hl = I.hl[s];
+        S.s = s;
+        S.in_sel = in_sel;
+        S.out_sel = out_sel;
+        S.terminator = I.terminator != 0;
+        S.wsc = static_cast<const R*>(I.wsc);
+        S.wstride = I.wstride;
+        it.lane = lane;
+#pragma unroll 1
+        for (int lb = set; lb * team_size + rank < nblk; lb += SETS) {
+          it.nb = lb * team_size + rank;
+          const R* src = S.win + (size_t)it.nb * (NN * 32);
+          if constexpr (STAGED) {
+            const int tid = sw * 32 + lane;
+            for (int i = tid; i < NN * 8; i += SW * 32) copy16_async(stage + 4 * i, src + 4 * i);
+            // the set's next block and this block's y on their way to L2
+            const int next = it.nb + SETS * team_size;
+            const char* pn = reinterpret_cast<const char*>(S.win + (size_t)next * (NN * 32));
+            const char* py = reinterpret_cast<const char*>(S.yv + (size_t)it.nb * (NN * 32));
+            for (int i = tid; i < NN; i += SW * 32) {
+              if (next < nblk) prefetch_l2(pn + 128 * i);
+              if (s != 0) prefetch_l2(py + 128 * i);
             }
+            asm volatile("cp.async.wait_all;" ::: "memory");
+            set_sync(1 + set, 32 * SW);
+            it.win = stage;
+          } else {
+            it.win = src;
           }
-          __syncthreads();
-          const int n = n0 + node;
-          if (n >= I.M) continue;
-          const bool root = (n == 0);
-          const R ng = ngam[n];
-          const bool term = I.terminator && I.up[n] < 0;
-          // packed element (i, j) of this lane's node; 0 outside the N x N matrix
-          auto Pk = [&](int i, int j) -> R { return (i < N && j < N) ? tile[(i * N + j) * TN + node] : R(0); };
-          // Re sigma_ij and Im sigma_ij (FULL tile: no bounds checks, padding is 0)
-          auto Sf = [&](int i, int j) -> R { return tile[(i * JS + j) * TN + node]; };
-          auto Af = [&](int i, int j) -> R { return tileA[(i * JS + j) * TN + node]; };
-          auto Re_ = [&](int i, int j) -> R { return FULL ? Sf(i, j) : Pk(i <= j ? i : j, i <= j ? j : i); };
-          auto Im_ = [&](int i, int j) -> R {
-            return FULL ? Af(i, j) : (i < j ? Pk(j, i) : (i > j ? -Pk(i, j) : R(0)));
-          };
-          for (int bk = warp; bk < nblk; bk += nwarps) {
-            // block index -> (A0, B0), A0 <= B0; this lane's rows A0 + 2 half + {0, 1}
-            int ab = 0, rem = bk;
-            while (rem >= NB - ab) { rem -= NB - ab; ++ab; }
-            const int A0 = 4 * ab + 2 * half, B0 = 4 * (ab + rem);
-            // A diagonal block (the same for the whole warp) keeps only its 10 entries
-            // with b >= a: in FP64, whose pipe bounds this kernel, the two lanes of a
-            // node take rows {0, 3} and {1, 2} of it, five entries each, instead of rows
-            // {0, 1} and {2, 3} with eight products each (about 11 % of the product work
-            // of a 24-site node); FP32 is bound by the neighbour gathers and keeps the
-            // plain blocks
-            const bool dblk = sizeof(R) == 8 && rem == 0;
-            const int ra0 = dblk ? 4 * ab + half : A0, ra1 = dblk ? 4 * ab + 3 - half : A0 + 1;
-            R re[2][4], im[2][4];
-            R rd[5], id[5];
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-              for (int j = 0; j < 4; ++j) re[i][j] = im[i][j] = R(0);
-#pragma unroll
-            for (int e = 0; e < 5; ++e) rd[e] = id[e] = R(0);
-            // -i[H, sigma] with the real part J (symmetric) and imaginary part Ji (antisymmetric) of H:
-            //   Re += sum_k J(a,k) A(k,b) - A(a,k) J(k,b);  Im -= sum_k J(a,k) S(k,b) - S(a,k) J(k,b)
-            //   Re += sum_k Ji(a,k) S(k,b) - S(a,k) Ji(k,b); Im += sum_k Ji(a,k) A(k,b) - A(a,k) Ji(k,b)
-            // with S = Re sigma, A = Im sigma; J(a,k) = J(k,a) is read from row k.
-#pragma unroll 2
-            for (int k = 0; k < N; ++k) {
-              R ja[2], jb[4];
-              ja[0] = cf[L::J(N) + k * JS + ra0];
-              ja[1] = cf[L::J(N) + k * JS + ra1];
-              load_row<4>(cf + L::J(N) + k * JS + B0, jb);
-              R sak[2], aak[2], skb[4], akb[4];
-#pragma unroll
-              for (int i = 0; i < 2; ++i) {
-                sak[i] = Re_(i ? ra1 : ra0, k);
-                aak[i] = Im_(i ? ra1 : ra0, k);
-              }
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                skb[j] = Re_(B0 + j, k);    // S(k, b) = S(b, k)
-                akb[j] = -Im_(B0 + j, k);   // A(k, b) = -A(b, k)
-              }
-              if (dblk) {
-                // the five entries (row r, column c) of this lane, picked by selects:
-                // half 0: (0,0) (0,1) (0,2) (0,3) (1,3); half 1: (0,1) (0,2) (0,3) (1,2) (1,3)
-                const bool hf = half != 0;
-                const R J0[5] = {ja[0], ja[0], ja[0], hf ? ja[1] : ja[0], ja[1]};
-                const R S0[5] = {sak[0], sak[0], sak[0], hf ? sak[1] : sak[0], sak[1]};
-                const R A0v[5] = {aak[0], aak[0], aak[0], hf ? aak[1] : aak[0], aak[1]};
-                const R JB[5] = {hf ? jb[1] : jb[0], hf ? jb[2] : jb[1], hf ? jb[3] : jb[2], hf ? jb[2] : jb[3], jb[3]};
-                const R SB[5] = {hf ? skb[1] : skb[0], hf ? skb[2] : skb[1], hf ? skb[3] : skb[2], hf ? skb[2] : skb[3],
-                                 skb[3]};
-                const R AB[5] = {hf ? akb[1] : akb[0], hf ? akb[2] : akb[1], hf ? akb[3] : akb[2], hf ? akb[2] : akb[3],
-                                 akb[3]};
-#pragma unroll
-                for (int e = 0; e < 5; ++e) {
-                  rd[e] = fma(J0[e], AB[e], rd[e]);
-                  rd[e] = fma(-A0v[e], JB[e], rd[e]);
-                  id[e] = fma(-J0[e], SB[e], id[e]);
-                  id[e] = fma(S0[e], JB[e], id[e]);
-                }
-                if constexpr (CPLX) {
-                  R ia[2], ib[4];
-                  ia[0] = cf[L::Ji(N) + k * JS + ra0];
-                  ia[1] = cf[L::Ji(N) + k * JS + ra1];
-                  load_row<4>(cf + L::Ji(N) + k * JS + B0, ib);
-                  const R I0[5] = {ia[0], ia[0], ia[0], hf ? ia[1] : ia[0], ia[1]};
-                  const R IB[5] = {hf ? ib[1] : ib[0], hf ? ib[2] : ib[1], hf ? ib[3] : ib[2], hf ? ib[2] : ib[3], ib[3]};
-#pragma unroll
-                  for (int e = 0; e < 5; ++e) {
-                    rd[e] = fma(-I0[e], SB[e], rd[e]);
-                    rd[e] = fma(-S0[e], IB[e], rd[e]);
-                    id[e] = fma(-I0[e], AB[e], id[e]);
-                    id[e] = fma(-A0v[e], IB[e], id[e]);
-                  }
-                }
-                continue;
-              }
-              // explicit multiply-add chains: two FMAs per output and term (written as
-              // x += a*b - c*d the compiler keeps a separate multiply and add, 1.5x the
-              // FP64 instructions of this loop)
-#pragma unroll
-              for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                  re[i][j] = fma(ja[i], akb[j], re[i][j]);
-                  re[i][j] = fma(-aak[i], jb[j], re[i][j]);
-                  im[i][j] = fma(-ja[i], skb[j], im[i][j]);
-                  im[i][j] = fma(sak[i], jb[j], im[i][j]);
-                }
-              if constexpr (CPLX) {
-                R ia[2], ib[4];  // row k of Ji: Ji(k, a) = -Ji(a, k)
-                ia[0] = cf[L::Ji(N) + k * JS + ra0];
-                ia[1] = cf[L::Ji(N) + k * JS + ra1];
-                load_row<4>(cf + L::Ji(N) + k * JS + B0, ib);
-#pragma unroll
-                for (int i = 0; i < 2; ++i)
-#pragma unroll
-                  for (int j = 0; j < 4; ++j) {
-                    re[i][j] = fma(-ia[i], skb[j], re[i][j]);
-                    re[i][j] = fma(-sak[i], ib[j], re[i][j]);
-                    im[i][j] = fma(-ia[i], akb[j], im[i][j]);
-                    im[i][j] = fma(-aak[i], ib[j], im[i][j]);
-                  }
-              }
-            }
-            if (dblk) {
-              // the five entries into their places of the 2 x 4 block (rows ra0, ra1); the
-              // places not set hold entries with b < a, which the epilogue drops
-              const bool hf = half != 0;
-              re[0][0] = rd[0];
-              im[0][0] = id[0];
-              re[0][1] = hf ? rd[0] : rd[1];
-              im[0][1] = hf ? id[0] : id[1];
-              re[0][2] = hf ? rd[1] : rd[2];
-              im[0][2] = hf ? id[1] : id[2];
-              re[0][3] = hf ? rd[2] : rd[3];
-              im[0][3] = hf ? id[2] : id[3];
-              re[1][2] = rd[3];
-              im[1][2] = id[3];
-              re[1][3] = rd[4];
-              im[1][3] = id[4];
-            }
-            // links of the block's rows and columns
-            int ua[2], ub[4], da[2], db[4];
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-              const int a = q ? ra1 : ra0;
-              ua[q] = a < N ? I.up[a * Mp + n] : -1;
-              da[q] = a < N ? I.dn[a * Mp + n] : -1;
-            }
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const int b = B0 + q;
-              ub[q] = b < N ? I.up[b * Mp + n] : -1;
-              db[q] = b < N ? I.dn[b * Mp + n] : -1;
-            }
-            // terminator factors (n_j + 1) / (ngam + gamma_j) of the block's rows and columns (leaf nodes)
-            R tca[2], tcb[4];
-#pragma unroll
-            for (int q = 0; q < 2; ++q) tca[q] = R(0);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) tcb[q] = R(0);
-            if (term) {
-#pragma unroll
-              for (int q = 0; q < 2; ++q) {
-                const int a = min(q ? ra1 : ra0, N - 1);
-                tca[q] = ((da[q] < 0 ? R(0) : R(da[q] >> 24)) + R(1)) / (ng + cf[L::gam(N) + a]);
-              }
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                const int b = min(B0 + q, N - 1);
-                tcb[q] = ((db[q] < 0 ? R(0) : R(db[q] >> 24)) + R(1)) / (ng + cf[L::gam(N) + b]);
-              }
-            }
-            // Per row and pair of columns: the local, neighbour and terminator
-            // terms of two outputs and their y values are loaded before their
-            // stores.
-#pragma unroll
-            for (int ij = 0; ij < 4; ++ij) {
-              const int i = ij >> 1, j0 = 2 * (ij & 1);
-              R yr[4], yim[4];
-              const int a = i ? ra1 : ra0;
-              const int ac = a < N ? a : N - 1;  // clamped for addressing; outputs with a >= N are dropped
-              const R* sa = cf + L::site(N) + 4 * ac;
-              const R eps_a = sa[0], gh_a = sa[1], al_a = sa[2], be_a = sa[3];
-              R na = da[i] < 0 ? R(0) : R(da[i] >> 24);
-              const int dai = da[i] < 0 ? -1 : (da[i] & 0xFFFFFF);
-              R wua = R(1);  // up-link weight of row a (scaled hierarchy)
-              if constexpr (SC) {
-                wua = scaled_up(static_cast<const R*>(I.wsc), I.wstride, ac, na);
-                na = scaled_dn(static_cast<const R*>(I.wsc), I.wstride, ac, na);
-              }
-              const R ca = tca[i];
-#pragma unroll
-              for (int j = j0; j < j0 + 2; ++j) {
-                const int b = B0 + j;
-                const int bc = b < N ? b : N - 1;
-                const bool keep = a < N && b < N && b >= a;
-                const int pr = ac * N + bc, pi = bc * N + ac;
-                yr[j] = ld_global_or0(yv + (pr * Mp + n), keep);
-                yim[j] = ld_global_or0(yv + (pi * Mp + n), keep && a != b);
-                const R* sb = cf + L::site(N) + 4 * bc;
-                const R eps_b = sb[0], gh_b = sb[1], al_b = sb[2], be_b = sb[3];
-                const R x = Re_(a, b), yi = Im_(a, b);
-                const int dbj = db[j] < 0 ? -1 : (db[j] & 0xFFFFFF);
-                R nb = db[j] < 0 ? R(0) : R(db[j] >> 24);
-                R wub = R(1);
-                if constexpr (SC) {
-                  wub = scaled_up(static_cast<const R*>(I.wsc), I.wstride, bc, nb);
-                  nb = scaled_dn(static_cast<const R*>(I.wsc), I.wstride, bc, nb);
-                }
-                // up-couplings i V_j^x sigma_{n+e_j}: j = a gives +i, j = b gives -i
-                const R uar = ld_global_or0(win + (pr * Mp + ua[i]), keep && a != b && ua[i] >= 0);
-                const R uai = ld_global_or0(win + (pi * Mp + ua[i]), keep && a != b && ua[i] >= 0);
-                const R ubr = ld_global_or0(win + (pr * Mp + ub[j]), keep && a != b && ub[j] >= 0);
-                const R ubi = ld_global_or0(win + (pi * Mp + ub[j]), keep && a != b && ub[j] >= 0);
-                // down-couplings n_j theta_j sigma_{n-e_j}
-                const R dar = ld_global_or0(win + (pr * Mp + dai), keep && dai >= 0);
-                const R dai_ = ld_global_or0(win + (pi * Mp + dai), keep && a != b && dai >= 0);
-                const R dbr = ld_global_or0(win + (pr * Mp + dbj), keep && a != b && dbj >= 0);
-                const R dbi = ld_global_or0(win + (pi * Mp + dbj), keep && a != b && dbj >= 0);
-                R r = re[i][j], m = im[i][j];
-                if (a != b) {
-                  // the same terms as the small-N units, as multiply-add chains
-                  const R d = eps_a - eps_b;
-                  const R c = ng + gh_a + gh_b;
-                  r = fma(d, yi, r);
-                  r = fma(-c, x, r);
-                  m = fma(-d, x, m);
-                  m = fma(-c, yi, m);
-                  if constexpr (SC) {
-                    r = fma(wub, ubi, r);
-                    r = fma(-wua, uai, r);
-                    m = fma(wua, uar, m);
-                    m = fma(-wub, ubr, m);
-                  } else {
-                    r += ubi - uai;
-                    m += uar - ubr;
-                  }
-                  if (I.terminator) {
-                    const R cbf = tcb[j];
-                    r += ca * (-al_a * x - be_a * yi) + cbf * (-al_b * x + be_b * yi);
-                    m += ca * (-al_a * yi + be_a * x) + cbf * (-al_b * yi - be_b * x);
-                  }
-                  const R nbe_a = na * be_a, nal_a = na * al_a, nbe_b = nb * be_b, nal_b = nb * al_b;
-                  r = fma(nbe_a, dar, r);
-                  r = fma(-nal_a, dai_, r);
-                  r = fma(nbe_b, dbr, r);
-                  r = fma(nal_b, dbi, r);
-                  m = fma(nal_a, dar, m);
-                  m = fma(nbe_a, dai_, m);
-                  m = fma(nbe_b, dbi, m);
-                  m = fma(-nal_b, dbr, m);
-                } else {
-                  r -= (ng + R(2) * cf[L::gd(N) + ac]) * x;
-                  r += R(2) * na * be_a * dar;
-                }
-                re[i][j] = r;
-                im[i][j] = m;
-              }
-              // Horner update w = y + h r and the stores (root in float-float for mixed precision)
-#pragma unroll
-              for (int j = j0; j < j0 + 2; ++j) {
-                const int b = B0 + j;
-                if (a >= N || b >= N || b < a) continue;
-                const int pr = a * N + b, pi = b * N + a;
-                const R r = re[i][j], m = im[i][j];
-                if (MIXED && root) {
-                  if constexpr (MIXED) {
-                    if (a == b && s == 3) ea.add(I, a, P.root_in[pr]);
-                    if (a == b && s == 2) ea.add_xi(I, a, P.root_in[pr]);
-                    const FF wr = ff_axpy(P.root_y[pr], P.h, P.hl, r);
-                    P.root_out[pr] = wr;
-                    wout[pr * Mp] = wr.h;
-                    if (a != b) {
-                      const FF wi = ff_axpy(P.root_y[pi], P.h, P.hl, m);
-                      P.root_out[pi] = wi;
-                      wout[pi * Mp] = wi.h;
-                    } else if (s == 3 && I.out_pops && os.now) {
-                      I.out_pops[os.row * N + a] = ff_to_double(wr);
-                    }
-                  }
-                } else {
-                  if constexpr (!MIXED) {
-                    if (root && a == b && s == 3) ea.add(I, cfd, N, a, (double)Re_(a, a));
-                    if (root && a == b && s == 2) ea.add_xi(I, cfd, a, (double)Re_(a, a));
-                  }
-                  const R vr = yr[j] + h * r;
-                  wout[pr * Mp + n] = vr;
-                  if (a != b) {
-                    wout[pi * Mp + n] = yim[j] + h * m;
-                  } else if (root && s == 3 && I.out_pops && os.now) {
-                    I.out_pops[os.row * N + a] = (double)vr;
-                  }
-                }
-              }
-            }
+          it.ng = S.ngam[it.nb * 32 + lane];
+#pragma unroll 1
+          for (int b = sw; b < N; b += SW) {
+            const int up = I.up[b * I.Mpad + it.nb * 32 + lane], dn = I.dn[b * I.Mpad + it.nb * 32 + lane];
+            if (EVEN && 2 * b >= N) large_hand_over<N, R, CPLX, EVEN>(it, s_cf, jt, jti, b, up, dn, ex);
+            else large_hand_over<N, R, CPLX, false>(it, s_cf, jt, jti, b, up, dn, ex);
           }
+          set_sync(1 + set, 32 * SW);
+#pragma unroll 1
+          for (int b = sw; b < N; b += SW) {
+            const int up = I.up[b * I.Mpad + it.nb * 32 + lane], dn = I.dn[b * I.Mpad + it.nb * 32 + lane];
+            if (EVEN && 2 * b < N)
+              large_finish<N, R, MIXED, CPLX, EVEN>(I, it, s_cf, jt, jti, s_rates, b, up, dn, ex, s_rows, s_root);
+            else
+              large_finish<N, R, MIXED, CPLX, false>(I, it, s_cf, jt, jti, s_rates, b, up, dn, ex, s_rows, s_root);
+          }
+          set_sync(1 + set, 32 * SW);  // the set's areas are free again
         }
-        if (s == 2 && slot >= 0) ea.step_xi(I);
-        if (s == 3 && slot >= 0 && (os.now || t + 1 == I.nsteps)) ea.store(I, slot);
+        // lane 0 of the warps of rank 0, set 0 (which run the root's block) keep the sums of their columns
+        if (s == 3 && rank == 0 && set == 0 && lane == 0 && (s_rows.os.now || t + 1 == I.nsteps))
+          for (int b = sw; b < N; b += SW) s_rows.ea[b].store(I, b);
         if (!team_barrier(A, epoch)) return;
       }
-      if (os.now) rows.pending = os.row;
+      if (lead) {
+        if (s_rows.os.now) s_rows.rows.pending = s_rows.os.row++;
+        s_rows.os.now = t + 2 == I.out_every * s_rows.os.row;
+      }
       if (I.stop_trace > 0.0 && t + 1 < I.nsteps && stop_now<R, MIXED>(I, N, &s_stop)) {
-        if (slot >= 0) ea.store(I, slot);
+        if (rank == 0 && set == 0 && lane == 0)
+          for (int b = sw; b < N; b += SW) s_rows.ea[b].store(I, b);
         done = t + 1;
         if (!team_barrier(A, epoch)) return;
         break;
       }
     }
-    if (lead) finish_instance<R>(I, nslots, rows, done, orow, N, A.status);
+    if constexpr (MIXED) {
+      if (rank == 0)
+        for (int p = threadIdx.x; p < NN; p += blockDim.x) {
+          bool neg;
+          const FF w = s_root.w[0][root_index(N, p / N, p % N, &neg)];
+          static_cast<FF*>(I.y0)[p] = neg ? FF{-w.h, -w.l} : w;
+        }
+      if (!team_barrier(A, epoch)) return;
+    }
+    if (lead) finish_instance<R>(I, N, s_rows.rows, done, s_rows.os.row, N, A.status);
     if (!team_barrier(A, epoch)) return;
     if (lead) signal_done(I);
   }
-}
-
-__host__ __device__ constexpr int large_smem_bytes(int N, int rsize) {
-  // FP32: unpacked Re and Im tiles of (4 ceil(N/4))^2 x 16 nodes; FP64: the packed tile N^2 x 16
-  return rsize == 8 ? N * N * kLargeTile * 8 + CoefLayout<double>::bytes(N)
-                    : 2 * CoefLayout<float>::JS(N) * CoefLayout<float>::JS(N) * kLargeTile * 4 +
-                          CoefLayout<float>::bytes(N);
 }
 
 }  // namespace heom

@@ -189,7 +189,7 @@ __global__ void set_root_kernel(R* y, int Mpad, float2* y0, const double* rho, i
       v = rho[2 * (b * N + a) + 1];
     else
       v = rho[2 * (a * N + a)];
-    y[heom::state_elem(N, Mpad, p, 0)] = (R)v;
+    heom::state_put(y, N, p, 0, v);
     if (y0) y0[p] = to_ff(v);
   }
   if (p == 0)
@@ -207,7 +207,7 @@ __global__ void unpack_state_kernel(const R* y, int Mpad, int64_t M, int N, cons
   const int a = e / N, b = e - (e / N) * N;
   auto P = [&](int k, int l) -> double {
     if (n == 0 && y0) return (double)y0[k * N + l].x + (double)y0[k * N + l].y;
-    return (double)y[heom::state_elem(N, Mpad, k * N + l, n)];
+    return heom::state_get(y, N, k * N + l, n);
   };
   double re, im;
   if (a < b) {
@@ -240,7 +240,7 @@ __global__ void pack_state_kernel(const double* in, R* y, int Mpad, int64_t M, i
     v = m[2 * (b * N + a) + 1];
   else
     v = m[2 * (a * N + a)];
-  y[heom::state_elem(N, Mpad, p, n)] = (R)v;
+  heom::state_put(y, N, p, n, v);
   if (n == 0 && y0) y0[p] = to_ff(v);
 }
 
@@ -254,10 +254,9 @@ __global__ void node_max_kernel(const R* y, int Mpad, int64_t M, int N, double* 
   if (n >= M) return;
   double mx = 0.0;
   for (int a = 0; a < N; ++a) {
-    mx = fmax(mx, fabs((double)y[heom::state_elem(N, Mpad, a * N + a, n)]));
+    mx = fmax(mx, fabs(heom::state_get(y, N, a * N + a, n)));
     for (int b = a + 1; b < N; ++b) {
-      const double re = (double)y[heom::state_elem(N, Mpad, a * N + b, n)];
-      const double im = (double)y[heom::state_elem(N, Mpad, b * N + a, n)];
+      const double re = heom::state_get(y, N, a * N + b, n), im = heom::state_get(y, N, b * N + a, n);
       mx = fmax(mx, sqrt(re * re + im * im));
     }
   }
@@ -983,11 +982,10 @@ struct Engine {
     TRY(in->stage.alloc(2 * sizeof(double) * p.N * p.N, hooks));
     CUDA_TRY(cudaMemcpyAsync(in->coef.p, in->coef_host.data(), in->coef_host.size(), cudaMemcpyHostToDevice, stream));
     CUDA_TRY(cudaMemsetAsync(in->y.p, 0, arr, stream));
-    if (p.N <= heom::kMaxSmallN) {  // the block of zeros that ends each stage buffer
-      const size_t live = (size_t)p.N * p.N * in->Mpad * rsize();
-      CUDA_TRY(cudaMemsetAsync(in->wa.as<unsigned char>() + live, 0, arr - live, stream));
-      CUDA_TRY(cudaMemsetAsync(in->wb.as<unsigned char>() + live, 0, arr - live, stream));
-    }
+    // the block of zeros that ends each stage buffer
+    const size_t live = (size_t)p.N * p.N * in->Mpad * rsize();
+    CUDA_TRY(cudaMemsetAsync(in->wa.as<unsigned char>() + live, 0, arr - live, stream));
+    CUDA_TRY(cudaMemsetAsync(in->wb.as<unsigned char>() + live, 0, arr - live, stream));
     CUDA_TRY(cudaMemsetAsync(in->acc.p, 0, kAccDoubles * sizeof(double), stream));
     CUDA_TRY(cudaStreamSynchronize(stream));  // coef_host must outlive the copy
     inst.push_back(std::move(in));
@@ -1094,7 +1092,7 @@ struct Engine {
       d.K = in.K;
       d.M = (int32_t)in.M;
       d.Mpad = in.Mpad;
-      d.rstride = in.N <= heom::kMaxSmallN ? 32 : in.Mpad;
+      d.dstride = heom::diag_stride(in.N);
       d.complex_h = in.complex_h;
       d.terminator = in.terminator;
       d.up = in.tab->up.as<int32_t>();
@@ -1155,7 +1153,7 @@ struct Engine {
       std::vector<int>& ids = kv.second;
       if (g.N > heom::kMaxSmallN) {
         if (g.c.mode == 2) return fail(HEOM_EINVAL, "launch mode 2 supports at most %d sites", heom::kMaxSmallN);
-        g.dyn = heom::large_smem_bytes(g.N, (int)rsize());
+        g.dyn = heom::large_smem_bytes(g.N, (int)rsize(), g.cplx != 0);
       } else if (g.c.mode == 2) {
         int64_t Mmax = 0;
         for (int id : ids) Mmax = std::max<int64_t>(Mmax, inst[id]->M);
@@ -1400,7 +1398,7 @@ struct Engine {
   // N <= 8.
   const void* kernel_for(int N, int cplx, int sc, const LaunchCfg& c) const {
     if (c.mode == 3) return flow_kernel_shape(cplx != 0, N, c.team_ctas);
-    if (N > heom::kMaxSmallN) return c.mode == 2 ? nullptr : heom::large_kernel(prec == HEOM_FP64, cplx != 0, sc != 0);
+    if (N > heom::kMaxSmallN) return c.mode == 2 ? nullptr : heom::large_kernel(prec == HEOM_FP64, cplx != 0, N);
     if (c.mode == 2) return (prec == HEOM_FP64 || sc) ? nullptr : heom::smem_kernel(cplx != 0, c.G <= 2, N);
     return heom::engine_kernel(prec == HEOM_FP64, cplx != 0, c.G, N, sc != 0);
   }
@@ -1427,8 +1425,10 @@ struct Engine {
     block_shape(N, c, M, &links, &dyn);
     return dyn;
   }
-  // Threads per CTA of a launch of modes 0 to 2: the block asked for, or the throughput engine's sets for it.
+  // Threads per CTA of a launch of modes 0 to 2: the block asked for, the throughput engine's sets for it, or the
+  // large-N engine's only size.
   int cta_threads(int N, int sc, const LaunchCfg& c) const {
+    if (N > heom::kMaxSmallN) return heom::large_threads(N, (int)rsize());
     return block_engine(N, sc, c) ? 32 * N * heom::block_sets(N, (int)rsize(), c.block) : c.block;
   }
 
@@ -2023,7 +2023,7 @@ int heom_autotune(heom_ctx* ctx, int64_t trial_steps, double* best_us_per_step) 
   const double dt = 1.0;
   for (const LaunchCfg& c : cands) {
     e.cfg[in.N] = c;
-    const int dyn = large ? heom::large_smem_bytes(in.N, (int)e.rsize())
+    const int dyn = large ? heom::large_smem_bytes(in.N, (int)e.rsize(), in.complex_h != 0)
                     : c.mode == 2 ? heom::smem_dyn_bytes(in.N, Engine::smem_slice(in.M, c.team_ctas))
                     : Engine::block_engine(in.N, in.scaled, c) ? e.block_dyn(in.N, c, in.M)
                                                                : 0;
@@ -2455,7 +2455,7 @@ extern "C" int heom_propagate_static(const heom_params* params, const double* d_
   d.K = p.K;
   d.M = (int32_t)M;
   d.Mpad = Mpad;
-  d.rstride = 32;
+  d.dstride = heom::diag_stride(N);
   d.complex_h = complex_h;
   d.terminator = p.terminator;
   d.up = reinterpret_cast<const int32_t*>(base + o_up);
