@@ -94,7 +94,7 @@ struct LargeCoef {
 // What the columns of one item share.
 template <typename R>
 struct LargeItem {
-  StageArgs<R> S;
+  const StageArgs<R>& S;  // in shared memory, so that the columns have the registers
   const R* win;    // the block's stage input: in shared memory (FP32) or device memory
   int nb, lane;
   R ng;
@@ -272,17 +272,24 @@ __device__ __forceinline__ void large_finish(const Inst& I, const LargeItem<R>& 
   R* wd = S.wout + self + b * 32 + lane;
   R2* wp = reinterpret_cast<R2*>(S.wout + self + N * 32) + lane;
   const R2* pairs = reinterpret_cast<const R2*>(it.win + N * 32) + lane;
-  const R s0 = it.win[b * 32 + lane];
+  const R s0 = it.win[b * 32 + lane], y0 = yd[b * 32 + lane];
+  // every y of the column before the first store: one trip to memory, not one per pair (the compiler keeps the order
+  // of loads and stores that may meet)
+  R2 y[C::NR];
+  static_for<1, C::NR>([&](auto ic) {
+    constexpr int r = decltype(ic)::value;
+    y[r] = yp[((r - 1) * N + b) * 32];
+  });
   {
     R d = R(2) * c.acc[0].y;
     d -= (it.ng + R(2) * cf.gd[b]) * s0;
     if (root) br.acc[b] = (float)d;
-    *wd = yd[b * 32 + lane] + S.h * d;
+    *wd = y0 + S.h * d;
   }
   static_for<1, C::NR>([&](auto ic) {
     constexpr int r = decltype(ic)::value;
     const int k = (r - 1) * N + b;
-    const R2 o = ex[k * 32], v = pairs[k * 32], y = yp[k * 32];
+    const R2 o = ex[k * 32], v = pairs[k * 32];
     const R* sa = cf.site[b + r];
     const R w = sa[0] - sb[0], g = it.ng + (sa[1] + sb[1]);
     R re = c.acc[r].y + o.x;
@@ -295,7 +302,11 @@ __device__ __forceinline__ void large_finish(const Inst& I, const LargeItem<R>& 
       br.acc[N + 2 * k] = (float)re;
       br.acc[N + 2 * k + 1] = (float)im;
     }
-    wp[k * 32] = R2{y.x + S.h * re, y.y + S.h * im};
+    c.acc[r] = R2{re, im};
+  });
+  static_for<1, C::NR>([&](auto ic) {
+    constexpr int r = decltype(ic)::value;
+    wp[((r - 1) * N + b) * 32] = R2{y[r].x + S.h * c.acc[r].x, y[r].y + S.h * c.acc[r].y};
   });
   if (it.nb == 0) {
     __syncwarp();
@@ -343,6 +354,7 @@ __global__ void __launch_bounds__(large_threads(N, (int)sizeof(R)), 1) heom_larg
   __shared__ BlockRoot<MIXED ? N : 1> s_root;
   __shared__ BlockRows<N, R> s_rows;
   __shared__ Inst s_inst;
+  __shared__ StageArgs<R> s_stage;
   __shared__ int s_stop;
   typedef typename Coupling<R>::type JT;
   typedef typename Vec2<R>::type R2;
@@ -429,22 +441,25 @@ __global__ void __launch_bounds__(large_threads(N, (int)sizeof(R)), 1) heom_larg
         }
         int in_sel, out_sel;
         stage_buffers(s, in_sel, out_sel);
-        LargeItem<R> it;
-        StageArgs<R>& S = it.S;
-        S.win = static_cast<const R*>(in_sel == 0 ? I.y : (in_sel == 1 ? I.wa : I.wb));
-        S.wout = static_cast<R*>(out_sel == 0 ? I.y : (out_sel == 1 ? I.wa : I.wb));
-        S.yv = static_cast<const R*>(I.y);
-        S.ngam = static_cast<const R*>(I.ngam);
-        S.zero = (unsigned)(I.Mpad >> 5) * (NN * 32);
-        S.h = RS == 8 ? (R)I.hd[s] : (R)I.hh[s];
-        S.hl = I.hl[s];
-        S.s = s;
-        S.in_sel = in_sel;
-        S.out_sel = out_sel;
-        S.terminator = I.terminator != 0;
-        S.wsc = static_cast<const R*>(I.wsc);
-        S.wstride = I.wstride;
-        it.lane = lane;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+          s_stage.win = static_cast<const R*>(in_sel == 0 ? I.y : (in_sel == 1 ? I.wa : I.wb));
+          s_stage.wout = static_cast<R*>(out_sel == 0 ? I.y : (out_sel == 1 ? I.wa : I.wb));
+          s_stage.yv = static_cast<const R*>(I.y);
+          s_stage.ngam = static_cast<const R*>(I.ngam);
+          s_stage.zero = (unsigned)(I.Mpad >> 5) * (NN * 32);
+          s_stage.h = RS == 8 ? (R)I.hd[s] : (R)I.hh[s];
+          s_stage.hl = I.hl[s];
+          s_stage.s = s;
+          s_stage.in_sel = in_sel;
+          s_stage.out_sel = out_sel;
+          s_stage.terminator = I.terminator != 0;
+          s_stage.wsc = static_cast<const R*>(I.wsc);
+          s_stage.wstride = I.wstride;
+        }
+        __syncthreads();
+        const StageArgs<R>& S = s_stage;
+        LargeItem<R> it{s_stage, nullptr, 0, lane, R(0)};
 #pragma unroll 1
         for (int lb = set; lb * team_size + rank < nblk; lb += SETS) {
           it.nb = lb * team_size + rank;
