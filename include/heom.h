@@ -282,9 +282,10 @@ int heom_ctx_num_nodes(const heom_ctx* ctx, int64_t* out);
  * than one: real H and 4..8 sites only, HEOM_EUNSUPPORTED otherwise), which
  * lets a hierarchy of up to about 6800 nodes (N = 7) run with all CTAs
  * resident; with more than three (two at N = 8) the throughput engine of mode 1
- * runs in its place, which is faster there.  Mode 3 is the default for one
- * hierarchy of 256 nodes or more when all its CTAs fit on the GPU at once with
- * some number of nodes per thread (the fewest that fit).  block_threads: multiple of 32, 64..512
+ * runs in its place, which is faster there, and a hierarchy of at most 992
+ * packed reals (nodes * N * N; 480 in HEOM_FP64) runs in one CTA with a thread per
+ * real.  Mode 3 is the default for one hierarchy when all its CTAs fit on the
+ * GPU at once with some number of nodes per thread (the fewest that fit).  block_threads: multiple of 32, 64..512
  * (64..256 for HEOM_FP64, whose kernels are compiled for that register budget);
  * in mode 3 the CTA size, at most 384 with one node per thread and 256 with
  * more, of which every N(N+1)/2 threads make a row of team_ctas nodes (N = 7,

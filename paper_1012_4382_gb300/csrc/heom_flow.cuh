@@ -596,4 +596,244 @@ __global__ void __launch_bounds__(NPT == 1 ? kFlowMaxThreads : kFlowMaxThreadsMu
   if (lead) finish_instance<R>(I, N, rows, done, orow, N, A.status);
 }
 
+// ------------------------------------------------------- one CTA, all on chip
+//
+// Hierarchies whose N*N*M reals fit the threads of one CTA (flow_small_fits):
+// one thread per real, all three stage arrays in shared memory ([N*N][M], so a
+// warp reads consecutive words), the right-hand side of the thread's element
+// -- own-node terms and the six neighbour terms alike -- as one list of (place,
+// coefficient) in registers, and a __syncthreads per stage.  Nothing leaves the
+// SM during a call but the output rows.  The bound is latency: a dependent chain
+// of shared-memory loads and multiply-adds and the barrier; in FP64 the pipe (64
+// cycles per instruction and warp), which is why the real and imaginary parts
+// of a pair are separate threads, terms that are zero in a whole warp are
+// skipped, and the output rows (sums and conversions in double) are left to one
+// more warp.  us per step with a row every step, two sites, depth 4, FP64: 10.2 as
+// a cluster launch of the load views, 8.4 of the throughput engine, 3.4 here
+// with the rows written by the root's warp.
+template <int N, typename R, bool CPLX>
+__host__ __device__ constexpr int flow_small_terms() {
+  return (flow_nre(N, CPLX) > flow_nim(N, CPLX) ? flow_nre(N, CPLX) : flow_nim(N, CPLX)) + 6;
+}
+// In FP64 the CTA's FP64 units soon cost more than an exchange through L2.
+__host__ __device__ constexpr int flow_small_max(int rsize) { return rsize == 8 ? 480 : 992; }
+__host__ __device__ constexpr bool flow_small_fits(int N, int rsize, int64_t M) { return M * N * N <= flow_small_max(rsize); }
+
+template <int N, typename R, bool MIXED, bool CPLX>
+__global__ void __launch_bounds__(flow_small_max((int)sizeof(R)) + 32, 1) heom_small_kernel(FlowArgs A) {
+  constexpr int NN = N * N;
+  constexpr int NP = N * (N - 1) / 2;
+  constexpr int U = NP + N;
+  constexpr int NRE = flow_nre(N, CPLX), NIM = flow_nim(N, CPLX);
+  constexpr int NT = NRE > NIM ? NRE : NIM;
+  constexpr int T = NT + 6;
+  __shared__ R s_st[3][flow_small_max((int)sizeof(R))];  // y, wa, wb
+  __shared__ Inst s_inst;
+  __shared__ int s_stop;
+  __shared__ EtaAcc<R> s_ea[kMaxSmallN];
+  __shared__ FF s_trace_ff[kMaxSmallN];
+  __shared__ double s_trace_d[kMaxSmallN];
+  if (threadIdx.x == 0) {
+    s_inst = *A.inst;
+    s_stop = 0;
+  }
+  __syncthreads();
+  const Inst& I = s_inst;
+  const int M = I.M, Mp = I.Mpad;
+  const int t_el = threadIdx.x;  // p * M + n
+  const bool valid = t_el < NN * M;
+  const int p = valid ? t_el / M : 0, n = valid ? t_el - p * M : 0;
+  const int er = p / N, ec = p - er * N;
+  const int a = min(er, ec), b = max(er, ec);
+  const bool im = er > ec, pair = er != ec, root = valid && n == 0, diag_root = root && !pair;
+  const bool lead = threadIdx.x == blockDim.x - 32;  // of the warp without elements
+  // FP64: this owner's step factors of eta, loss and xi
+  double fe = 0.0, fl = 0.0, fx = 0.0;
+
+  // the element's list: NT own terms, then n + e_a, n + e_b, n - e_a (two), n - e_b (two)
+  R co[T];
+  unsigned pl[(T + 1) / 2];  // places, 16 bits each
+#pragma unroll
+  for (int i = 0; i < T; ++i) co[i] = R(0);
+#pragma unroll
+  for (int i = 0; i < (T + 1) / 2; ++i) pl[i] = (unsigned)t_el | ((unsigned)t_el << 16);
+  auto put = [&](auto ic, double w, int place) {
+    constexpr int i = decltype(ic)::value;
+    co[i] = (R)w;
+    pl[i / 2] = i % 2 ? (pl[i / 2] & 0xFFFFu) | ((unsigned)place << 16) : (pl[i / 2] & 0xFFFF0000u) | (unsigned)place;
+  };
+  if (!valid) {
+#pragma unroll
+    for (int i = 0; i < (T + 1) / 2; ++i) pl[i] = 0;
+  } else {
+    const int u = pair ? a * (2 * N - a - 1) / 2 + b - a - 1 : NP + a;
+    const FlowUnit& fu = A.units[u];
+    const FlowSite* fs = reinterpret_cast<const FlowSite*>(A.units + U);
+    const FlowSite sa = fs[a], sb = fs[b];
+    const bool scaled = I.wsc != nullptr;
+    const int pab = a * N + b, pba = b * N + a;
+    const int ra = I.dn[a * Mp + n], rb = I.dn[b * Mp + n], ua = I.up[a * Mp + n], ub = I.up[b * Mp + n];
+    const double na = ra < 0 ? 0.0 : (double)(ra >> 24), nb = rb < 0 ? 0.0 : (double)(rb >> 24);
+    const double ng = (double)static_cast<const R*>(I.ngam)[n];
+    // terms of the node itself on x (slot 0) and, for a pair, yi (slot 1): hierarchy damping and the terminator (see
+    // heom_flow_kernel)
+    double x0 = im ? 0.0 : -ng, x1 = im ? -ng : 0.0;
+    if (pair && I.terminator && I.up[n] < 0) {
+      const double ca = (na + 1.0) / (ng + sa.gamma), cb = (nb + 1.0) / (ng + sb.gamma);
+      const double re = -ca * sa.alpha - cb * sb.alpha, ro = -ca * sa.beta + cb * sb.beta;
+      x0 += im ? -ro : re;
+      x1 += im ? re : ro;
+    }
+    static_for<0, NT>([&](auto ic) {
+      constexpr int i = decltype(ic)::value;
+      const bool in = im ? i < NIM : i < NRE;
+      if (!in) return;
+      double w = im ? fu.cim[i < NIM ? i : 0] : fu.cre[i < NRE ? i : 0];
+      if (i == 0) w += x0;
+      if (i == 1 && pair) w += x1;
+      put(ic, w, (im ? fu.iim[i < NIM ? i : 0] : fu.ire[i < NRE ? i : 0]) * M + n);
+    });
+    const double wua = scaled ? sqrt((na + 1.0) * sa.scale) : 1.0, wub = scaled ? sqrt((nb + 1.0) * sb.scale) : 1.0;
+    const double wa = scaled ? sqrt(na / sa.scale) : na, wb = scaled ? sqrt(nb / sb.scale) : nb;
+    const int da = ra & 0xFFFFFF, db = rb & 0xFFFFFF;
+    if (pair) {
+      // re: -wu_a Im(up a) + wu_b Im(up b); im: wu_a Re(up a) - wu_b Re(up b)
+      if (ua >= 0) put(std::integral_constant<int, NT>{}, im ? wua : -wua, (im ? pab : pba) * M + ua);
+      if (ub >= 0) put(std::integral_constant<int, NT + 1>{}, im ? -wub : wub, (im ? pab : pba) * M + ub);
+      // n_j theta_j: re: beta Re -+ alpha Im, im: beta Im +- alpha Re (upper sign for j = a)
+      if (ra >= 0) {
+        put(std::integral_constant<int, NT + 2>{}, wa * sa.beta, p * M + da);
+        put(std::integral_constant<int, NT + 3>{}, im ? wa * sa.alpha : -wa * sa.alpha, (im ? pab : pba) * M + da);
+      }
+      if (rb >= 0) {
+        put(std::integral_constant<int, NT + 4>{}, wb * sb.beta, p * M + db);
+        put(std::integral_constant<int, NT + 5>{}, im ? -wb * sb.alpha : wb * sb.alpha, (im ? pab : pba) * M + db);
+      }
+    } else if (ra >= 0) {
+      put(std::integral_constant<int, NT + 2>{}, 2.0 * wa * sa.beta, p * M + da);
+    }
+  }
+  uint64_t terms = 0;  // terms some lane of the warp has
+#pragma unroll
+  for (int i = 0; i < T; ++i) terms |= __any_sync(0xFFFFFFFFu, co[i] != R(0)) ? 1ull << i : 0ull;
+
+  R y = R(0);
+  FF ry{0.f, 0.f}, rw{0.f, 0.f};  // the root's element in float-float: y and the last stage output (mixed)
+  if (valid) {
+    y = static_cast<const R*>(I.y)[node_col<N>(n) + p * 32];
+    s_st[0][t_el] = y;
+    if constexpr (MIXED) {
+      if (root) ry = static_cast<const FF*>(I.y0)[p];
+    }
+  }
+  if (diag_root) s_ea[a] = EtaAcc<R>{};
+  EtaRows rows;
+  rows.acc0 = I.acc[0];
+  rows.acc1 = I.acc[1];
+  const double* cfd = reinterpret_cast<const double*>(static_cast<const unsigned char*>(I.coef) +
+                                                      CoefLayout<R>::dbl_offset(N));
+  if (diag_root) {
+    fe = I.dt * cfd[a];
+    fl = I.dt * cfd[N + a];
+    fx = 0.5 * I.dt * I.dt * cfd[a];
+  }
+  if (lead) {
+    write_row0<N, R, MIXED>(I);
+    const EtaAcc<R> zero{};
+    for (int k = 0; k < N; ++k) zero.store(I, k);
+  }
+  __syncthreads();
+
+  int64_t next_out = I.out_every, orow = 1, done = I.nsteps;
+  for (int64_t t = 0; t < I.nsteps; ++t) {
+    const OutStep os{t + 1 == next_out, orow};
+    if (os.now) {
+      next_out += I.out_every;
+      ++orow;
+    }
+#pragma unroll 1
+    for (int s = 0; s < 4; ++s) {
+      if (s == 0 && rows.pending >= 0) {
+        if (lead) flow_eta_row<R, MIXED>(I, s_ea, s_trace_ff, s_trace_d, N, rows.acc0, rows.acc1, rows.pending, A.status);
+        rows.pending = -1;
+      }
+      const R* sin = s_st[s == 0 ? 0 : (s == 2 ? 2 : 1)];
+      R* sout = s_st[s == 1 ? 2 : (s == 3 ? 0 : 1)];
+      R r0 = R(0), r1 = R(0);
+#pragma unroll
+      for (int i = 0; i < T; ++i) {
+        if (sizeof(R) == 8 && !((terms >> i) & 1)) continue;
+        const R v = sin[(pl[i / 2] >> (16 * (i % 2))) & 0xFFFFu];
+        if (i % 2) r1 += co[i] * v;
+        else r0 += co[i] * v;
+      }
+      const R r = r0 + r1;
+      if (valid) {
+        R w;
+        if (MIXED && root) {
+          if constexpr (MIXED) {
+            if (diag_root) {
+              if (s == 3) s_ea[a].add(I, a, rw);
+              if (s == 2) s_ea[a].add_xi(I, a, rw);
+            }
+            rw = ff_axpy(ry, I.hh[s], I.hl[s], r);
+            w = rw.h;
+            if (s == 3) {
+              ry = rw;
+              if (diag_root && os.now && I.out_pops) I.out_pops[os.row * N + a] = ff_to_double(rw);
+            }
+          }
+        } else {
+          if constexpr (!MIXED) {
+            if (diag_root && s == 3) {
+              s_ea[a].e += fe * sin[t_el];
+              s_ea[a].l += fl * sin[t_el];
+            }
+            if (diag_root && s == 2) s_ea[a].x += fx * sin[t_el];
+          }
+          w = y + (sizeof(R) == 8 ? (R)I.hd[s] : (R)I.hh[s]) * r;
+          if (diag_root && s == 3 && os.now && I.out_pops) I.out_pops[os.row * N + a] = (double)w;
+        }
+        sout[t_el] = w;
+        if (s == 3) y = w;
+        if (diag_root) {
+          if (s == 2) s_ea[a].step_xi(I);
+          if (s == 3) {
+            if (os.now || t + 1 == I.nsteps) s_ea[a].store(I, a);
+            if constexpr (MIXED) s_trace_ff[a] = ry;
+            else s_trace_d[a] = (double)w;
+          }
+        }
+      }
+      __syncthreads();
+    }
+    if (os.now) rows.pending = os.row;
+    if (I.stop_trace > 0.0 && t + 1 < I.nsteps) {
+      if (lead) {
+        double tr = 0.0;
+        if constexpr (MIXED) {
+          FF sum{0.f, 0.f};
+          for (int k = 0; k < N; ++k) sum = ff_add(sum, s_trace_ff[k]);
+          tr = ff_to_double(sum);
+        } else {
+          for (int k = 0; k < N; ++k) tr += s_trace_d[k];
+        }
+        s_stop = tr < I.stop_trace;
+      }
+      __syncthreads();
+      if (s_stop) {
+        if (diag_root) s_ea[a].store(I, a);
+        done = t + 1;
+        break;
+      }
+    }
+  }
+  if (valid) static_cast<R*>(I.y)[node_col<N>(n) + p * 32] = y;
+  if constexpr (MIXED) {
+    if (root) static_cast<FF*>(I.y0)[p] = ry;
+  }
+  __syncthreads();
+  if (lead) finish_instance<R>(I, N, rows, done, orow, N, A.status);
+}
+
 }  // namespace heom

@@ -35,6 +35,12 @@ const void* flow_kernel_f64(int N, bool cplx, int npt);
 inline const void* flow_kernel(bool fp64, bool cplx, int N, int npt = 1) {
   return fp64 ? flow_kernel_f64(N, cplx, npt) : flow_kernel_f32(N, cplx, npt);
 }
+// One CTA with a thread per real of the hierarchy, N = 1..8 (mode 3 on small hierarchies).
+const void* small_kernel_f32(int N, bool cplx);
+const void* small_kernel_f64(int N, bool cplx);
+inline const void* small_kernel(bool fp64, bool cplx, int N) {
+  return fp64 ? small_kernel_f64(N, cplx) : small_kernel_f32(N, cplx);
+}
 // Distributed-shared-memory engine (mixed precision only).
 const void* smem_kernel_f32_real(int N, bool reg);
 const void* smem_kernel_f32_cplx(int N, bool reg);

@@ -37,4 +37,19 @@ const void* flow_kernel_f64(int N, bool cplx, int npt) {
   }
 }
 
+// One CTA, one thread per real.
+const void* small_kernel_f64(int N, bool cplx) {
+  switch (N) {
+    case 1: return cplx ? (const void*)heom_small_kernel<1, double, false, true> : (const void*)heom_small_kernel<1, double, false, false>;
+    case 2: return cplx ? (const void*)heom_small_kernel<2, double, false, true> : (const void*)heom_small_kernel<2, double, false, false>;
+    case 3: return cplx ? (const void*)heom_small_kernel<3, double, false, true> : (const void*)heom_small_kernel<3, double, false, false>;
+    case 4: return cplx ? (const void*)heom_small_kernel<4, double, false, true> : (const void*)heom_small_kernel<4, double, false, false>;
+    case 5: return cplx ? (const void*)heom_small_kernel<5, double, false, true> : (const void*)heom_small_kernel<5, double, false, false>;
+    case 6: return cplx ? (const void*)heom_small_kernel<6, double, false, true> : (const void*)heom_small_kernel<6, double, false, false>;
+    case 7: return cplx ? (const void*)heom_small_kernel<7, double, false, true> : (const void*)heom_small_kernel<7, double, false, false>;
+    case 8: return cplx ? (const void*)heom_small_kernel<8, double, false, true> : (const void*)heom_small_kernel<8, double, false, false>;
+    default: return nullptr;
+  }
+}
+
 }  // namespace heom

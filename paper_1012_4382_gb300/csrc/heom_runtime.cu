@@ -386,6 +386,7 @@ struct LaunchCfg {
   int team_ctas = 1;
   int block = 256;
   int G = 1;
+  bool automatic = false;  // the default of one hierarchy under 256 nodes, until a launch shape is set
 };
 
 int ilog2(int v) {
@@ -731,6 +732,7 @@ struct Engine {
   std::vector<std::unique_ptr<Instance>> inst;
   std::shared_ptr<TableCache> tables = std::make_shared<TableCache>();
   std::map<int, LaunchCfg> cfg;  // per N
+  bool batch = false;             // made by heom_batch_create*
   double stop_trace = 0.0;        // the stop rule (0: off)
   const uint8_t* subset_keep = nullptr;  // while a filtered context is created: its node flags
   const uint8_t* const* subset_keeps = nullptr;  // while a filtered batch is created: per instance (may hold NULL)
@@ -874,9 +876,10 @@ struct Engine {
       }
       return c;
     }
-    if (count == 1) {
-      // one hierarchy of 256 nodes or more: the dataflow engine (mode 3), when all its
-      // CTAs fit on the GPU at once.  Nodes per CTA, measured on the FMO-like N = 7,
+    // (a batch of one small hierarchy keeps a shape that CUDA graphs take)
+    if (count == 1 && !(batch && Mmax < 256)) {
+      // one hierarchy: the dataflow engine (mode 3), when all its CTAs fit on the GPU at
+      // once (small ones in one CTA, see heom_small_kernel).  Nodes per CTA, measured on the FMO-like N = 7,
       // depth 6 hierarchy and a filtered version of it (1225 nodes): in mixed precision
       // CTAs of about 336 threads (12 nodes at N = 7: 1.25 us per stage for both, 1.45-2.3
       // with 5-11 or 13 nodes); in FP64, bound by the FP64 pipe, the nodes spread evenly
@@ -885,7 +888,7 @@ struct Engine {
       // carries npt = 2..6 nodes of its unit (real H, N >= 4; CTAs of at most 256 threads,
       // the nodes spread evenly): the fewest nodes per thread with which all CTAs fit
       // (launch_flow says what runs with more than three).
-      if (Mmax >= 256) {
+      {
         const int U = N * (N + 1) / 2;
         bool cplx_any = false;
         for (auto& in : inst) cplx_any |= (in->N == N && in->complex_h);
@@ -905,28 +908,17 @@ struct Engine {
             c.block = S * U;
             c.G = 1;
             c.team_ctas = npt;
+            c.automatic = Mmax < 256;
             return c;
           }
           cudaGetLastError();
         }
       }
-      if ((prec == HEOM_FP64 && Mmax >= 256) || (prec == HEOM_FP32_MIXED && Mmax >= 1024)) {
-        // the throughput engine on the whole grid
-        c.mode = 1;
-        c.team_ctas = 1;
-        c.block = max_block();
-        c.G = 2;
-      } else {
-        // small: the throughput engine in one CTA while its blocks of 32 nodes fill at most one round of sets, else
-        // in a cluster with a block per CTA
-        c.mode = 0;
-        c.block = max_block();
-        c.G = 2;
-        const int64_t nb = (Mmax + 31) / 32;
-        c.team_ctas = 1;
-        if (nb > heom::block_sets(N, (int)rsize(), c.block))
-          while (c.team_ctas < 16 && c.team_ctas < nb) c.team_ctas <<= 1;
-      }
+      // larger: the throughput engine on the whole grid
+      c.mode = 1;
+      c.team_ctas = 1;
+      c.block = max_block();
+      c.G = 2;
     } else {
       // many hierarchies: the throughput engine with the team size batch_team picks.  Keeping small hierarchies in
       // shared memory (mode 2) loses to it: 64 hierarchies of 70 nodes (N = 4) 14.9 us a step against 7.2, 300 of 252
@@ -1377,7 +1369,7 @@ struct Engine {
   // The dataflow kernel that stands for npt nodes per thread: the built one, and for more (mixed precision) the largest built,
   // which takes the same registers per thread and so has the same residency.  nullptr: not supported.
   const void* flow_kernel_shape(bool cplx, int N, int npt) const {
-    if (N > heom::kMaxSmallN || npt < 1 || npt > heom::kFlowMaxNpt) return nullptr;
+    if (N > heom::kMaxSmallN || npt < 1 || npt > (prec == HEOM_FP64 ? 2 : heom::kFlowMaxNpt)) return nullptr;
     return heom::flow_kernel(prec == HEOM_FP64, cplx, N, std::min(npt, heom::flow_built_npt(N)));
   }
 
@@ -1428,13 +1420,29 @@ struct Engine {
       block_shape(N, g, in.M, &links, &bytes);
       return launch(N, in.complex_h, in.scaled, g, 1, A, links, bytes);
     }
-    const long long wd = fp64 ? 2 : 1;
-    const long long stride = (long long)NN * in.Mpad * wd;
-    if (!in.flow_tags.p) {
+    if (!in.flow_units.p) {
       std::vector<unsigned char> tab;
       TRY(flow_table(in, tab));
       TRY(in.flow_units.alloc(tab.size(), hooks));
       CUDA_TRY(cudaMemcpy(in.flow_units.p, tab.data(), tab.size(), cudaMemcpyHostToDevice));
+    }
+    heom::FlowArgs F;
+    F.inst = d_inst;
+    F.units = in.flow_units.as<heom::FlowUnit>();
+    F.status = A.status;
+    F.S = S;
+    if (heom::flow_small_fits(N, (int)rsize(), in.M)) {
+      F.tags = F.ring = nullptr;
+      F.tag_stride = 0;
+      F.tag0 = 0;
+      const int small = (int)((in.M * NN + 31) / 32 * 32) + 32;  // and the warp that writes the rows
+      void* sargs[] = {&F};
+      CUDA_TRY(cudaLaunchKernel(heom::small_kernel(fp64, in.complex_h != 0, N), dim3(1), dim3(small), sargs, 0, stream));
+      return HEOM_OK;
+    }
+    const long long wd = fp64 ? 2 : 1;
+    const long long stride = (long long)NN * in.Mpad * wd;
+    if (!in.flow_tags.p) {
       TRY(in.flow_tags.alloc(sizeof(unsigned long long) * (3 * stride + heom::kFlowRing), hooks));
       CUDA_TRY(cudaMemsetAsync(in.flow_tags.p, 0, in.flow_tags.bytes, stream));
       in.flow_tag = 0;
@@ -1445,14 +1453,9 @@ struct Engine {
       CUDA_TRY(cudaMemsetAsync(in.flow_tags.p, 0, in.flow_tags.bytes, stream));
       in.flow_tag = 0;
     }
-    heom::FlowArgs F;
-    F.inst = d_inst;
-    F.units = in.flow_units.as<heom::FlowUnit>();
     F.tags = in.flow_tags.as<unsigned long long>();
     F.tag_stride = stride;
     F.ring = F.tags + 3 * stride;
-    F.status = A.status;
-    F.S = S;
     F.tag0 = in.flow_tag;
     in.flow_tag += need;
     void* args[] = {&F};
@@ -1957,7 +1960,16 @@ int heom_ctx_num_nodes(const heom_ctx* ctx, int64_t* out) {
 int heom_set_launch(heom_ctx* ctx, int32_t mode, int32_t team_ctas, int32_t block_threads, int32_t node_threads) {
   if (!ctx) return fail(HEOM_EINVAL, "ctx is NULL");
   LaunchCfg& c = ctx->e.cfg[ctx->e.inst[0]->N];
+  if (c.automatic && mode < 0 && (team_ctas > 0 || block_threads > 0 || node_threads > 0)) {
+    // team_ctas, block_threads or node_threads alone, on a small hierarchy whose shape was never set: they are those of
+    // a cluster launch, as they mean nothing to the one-CTA kernel the default runs
+    c.mode = 0;
+    c.team_ctas = 1;
+    c.block = ctx->e.max_block();
+    c.G = ctx->e.inst[0]->scaled ? 4 : 2;
+  }
   LaunchCfg n = c;
+  n.automatic = false;
   if (mode >= 0) n.mode = mode;
   if (team_ctas > 0) n.team_ctas = team_ctas;
   if (block_threads > 0) n.block = block_threads;
@@ -2127,6 +2139,7 @@ int heom_batch_create(const heom_params* params, int32_t count, void* cuda_strea
   if (!out) return fail(HEOM_EINVAL, "out is NULL");
   *out = nullptr;
   auto b = std::make_unique<heom_batch>();
+  b->e.batch = true;
   TRY(b->e.init(params, count, cuda_stream));
   *out = b.release();
   return HEOM_OK;
@@ -2142,6 +2155,7 @@ int heom_batch_create_subset(const heom_params* params, const uint8_t* const* ke
     if (keep[i] && params[i].terminator != HEOM_TERM_NONE)
       return fail(HEOM_EUNSUPPORTED, "params[%d]: a filtered hierarchy takes the plain truncation", i);
   auto b = std::make_unique<heom_batch>();
+  b->e.batch = true;
   b->e.subset_keeps = keep;
   const int rc = b->e.init(params, count, cuda_stream);
   b->e.subset_keeps = nullptr;
