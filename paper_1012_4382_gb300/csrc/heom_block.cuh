@@ -115,7 +115,7 @@ struct StageArgs {
   R* wout;
   const R* yv;
   const R* ngam;
-  unsigned zero;  // the zero block
+  unsigned zero;  // the zero block: its first element (N > 8: its index)
   R h;
   float hl;       // low part of h (mixed)
   int s, in_sel, out_sel;

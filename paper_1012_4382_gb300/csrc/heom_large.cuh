@@ -22,6 +22,18 @@
 // four times; FP64, bound by its pipe, reads it through L1.  Links that no lane
 // of the warp has (most: a node of depth 4 has at most four nonzero n_j) are
 // skipped by a vote, with their arithmetic.
+//
+// Bound and measured (24 sites, depth 4, 20 475 nodes, whole grid; in brackets
+// the kernel this one took the place of, 4x4 blocks of 16 nodes with two lanes
+// a node): mixed precision 80 us per stage [148], bound by issue slots and the
+// barriers between the phases of the one block an SM holds; FP64 1304 us [1800],
+// bound by the FP64 pipe (the algorithm's multiply-adds alone 1000 us).  16
+// sites, mixed: 9.8 us [21] at depth 4, 29.5 [66] at depth 5.  What made the
+// difference in FP32, us per stage: y of a column read in one batch (a load
+// between two stores waits for its own round trip) and the stage's arguments in
+// shared memory instead of registers, 92 -> 80.  Tried and dropped: two columns
+// a warp with absolute rows and a table of places 117 to 136, two columns with
+// relative rows 105, the same with the staged block 99.5, rows in halves 102.
 #pragma once
 
 #include "heom_block.cuh"
@@ -184,7 +196,8 @@ struct HalfColumn {
       w_up = scaled_up(S.wsc, S.wstride, b, n_b);
       w_dn = scaled_dn(S.wsc, S.wstride, b, n_b);
     }
-    auto linked = [&](int l) { return S.win + (size_t)(l >= 0 ? (unsigned)(l >> 5) * (N * N * 32) : S.zero); };
+    // (the elements of a state may pass 2^32: 24 sites from depth 8)
+    auto linked = [&](int l) { return S.win + (size_t)(l >= 0 ? (unsigned)(l >> 5) : S.zero) * (N * N * 32); };
     if (__any_sync(0xFFFFFFFFu, dn >= 0)) {
       const int m = dn < 0 ? -1 : (dn & 0xFFFFFF);
       const R* g0 = linked(m) + (m & 31);
@@ -447,7 +460,7 @@ __global__ void __launch_bounds__(large_threads(N, (int)sizeof(R)), 1) heom_larg
           s_stage.wout = static_cast<R*>(out_sel == 0 ? I.y : (out_sel == 1 ? I.wa : I.wb));
           s_stage.yv = static_cast<const R*>(I.y);
           s_stage.ngam = static_cast<const R*>(I.ngam);
-          s_stage.zero = (unsigned)(I.Mpad >> 5) * (NN * 32);
+          s_stage.zero = (unsigned)(I.Mpad >> 5);
           s_stage.h = RS == 8 ? (R)I.hd[s] : (R)I.hh[s];
           s_stage.hl = I.hl[s];
           s_stage.s = s;
