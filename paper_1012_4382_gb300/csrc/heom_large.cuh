@@ -15,7 +15,7 @@
 // the exchanged elements and the local terms, and stored.  So a thread holds
 // the accumulators of half a column (26 registers in FP32, 52 in FP64 at N =
 // 24), and every coupling read from shared memory (a broadcast) serves two
-// multiply-adds, in FP32 one packed instruction.
+// multiply-adds, in FP32 packed two rows to an instruction (fma.rn.f32x2).
 //
 // FP32 first brings the block's stage input (74 KB at N = 24) into shared
 // memory, since the two phases and the two columns of a pair read every element
@@ -25,15 +25,18 @@
 //
 // Bound and measured (24 sites, depth 4, 20 475 nodes, whole grid; in brackets
 // the kernel this one took the place of, 4x4 blocks of 16 nodes with two lanes
-// a node): mixed precision 80 us per stage [148], bound by issue slots and the
-// barriers between the phases of the one block an SM holds; FP64 1304 us [1800],
-// bound by the FP64 pipe (the algorithm's multiply-adds alone 1000 us).  16
-// sites, mixed: 9.8 us [21] at depth 4, 29.5 [66] at depth 5.  What made the
-// difference in FP32, us per stage: y of a column read in one batch (a load
-// between two stores waits for its own round trip) and the stage's arguments in
-// shared memory instead of registers, 92 -> 80.  Tried and dropped: two columns
-// a warp with absolute rows and a table of places 117 to 136, two columns with
-// relative rows 105, the same with the staged block 99.5, rows in halves 102.
+// a node): mixed precision 70 us per stage [148], bound by issue slots, shared
+// memory and the barriers between the phases of the one block an SM holds; FP64
+// 1300 us [1800], bound by the FP64 pipe (the algorithm's multiply-adds alone
+// 1000 us).  16 sites, mixed: 9.2 us [21] at depth 4, 27.3 [66] at depth 5.
+// What made the difference in FP32, us per stage: y of a column read in one
+// batch (a load between two stores waits for its own round trip) and the stage's
+// arguments in shared memory instead of registers, 92 -> 80; two rows instead of
+// the two parts of one row per packed multiply-add, which halves the bytes of
+// couplings read (a broadcast 16-byte read takes two passes of the shared-memory
+// pipe), 80 -> 70.  Tried and dropped: two columns a warp with absolute rows and
+// a table of places 117 to 136, two columns with relative rows 105, the same
+// with the staged block 99.5, rows in halves 102.
 #pragma once
 
 #include "heom_block.cuh"
@@ -48,44 +51,81 @@ __host__ __device__ constexpr int large_sets(int N, int rsize) { return N <= (rs
 __host__ __device__ constexpr int large_threads(int N, int rsize) {
   return 32 * large_set_warps(N, rsize) * large_sets(N, rsize);
 }
-// Coupling table: two copies (the second shifted by one entry, so that a row's
-// part can be read two entries at a time from any column) of [N][2N] entries of
-// 8 bytes: a double, or a float twice.
-__host__ __device__ constexpr int large_jrow(int N) { return 2 * N + 4; }
-__host__ __device__ constexpr int large_jbytes(int N) { return 2 * N * large_jrow(N) * 8; }
+// Coupling table [copy][N][jrow]: one copy per entry of a 16-byte word, each
+// shifted by one entry more, so that a row's part starts a word in one of them
+// from any column.
+__host__ __device__ constexpr int large_jcopies(int rsize) { return 16 / rsize; }
+__host__ __device__ constexpr int large_jrow(int N, int rsize) {
+  const int w = large_jcopies(rsize);
+  return (2 * N + 2 * w + w - 1) / w * w;  // columns to 2N - 2, the shift and the last word's rest
+}
+__host__ __device__ constexpr int large_jbytes(int N, int rsize) {
+  return large_jcopies(rsize) * N * large_jrow(N, rsize) * rsize;
+}
 __host__ __device__ constexpr int large_stage_bytes(int N, int rsize) { return rsize == 4 ? N * N * 32 * 4 : 0; }
 __host__ __device__ constexpr int large_exch_bytes(int N, int rsize) { return N * (N - 1) * 32 * rsize; }
 __host__ __device__ constexpr int large_smem_bytes(int N, int rsize, bool cplx) {
-  return (cplx ? 2 : 1) * large_jbytes(N) +
+  return (cplx ? 2 : 1) * large_jbytes(N, rsize) +
          large_sets(N, rsize) * (large_stage_bytes(N, rsize) + large_exch_bytes(N, rsize));
 }
 
-// A coupling entry and its multiply-add on a complex accumulator.
-template <typename R>
-struct Coupling;
-template <>
-struct Coupling<double> {
-  typedef double type;
-  static __device__ __forceinline__ double make(double v) { return v; }
-  static __device__ __forceinline__ void fma2(double2& acc, double j, double2 v) {
-    acc.x = fma(j, v.x, acc.x);
-    acc.y = fma(j, v.y, acc.y);
+// The sum over k of J(k, row) sigma_k for NR rows: j holds NR couplings (and
+// what fills the last 16-byte word), x and y multiply them into the real and
+// imaginary sums.
+template <typename R, int NR>
+struct ColumnSum;
+template <int NR>
+struct ColumnSum<double, NR> {
+  double re[NR], im[NR];
+  __device__ __forceinline__ ColumnSum() {
+#pragma unroll
+    for (int i = 0; i < NR; ++i) re[i] = im[i] = 0.0;
   }
-};
-template <>
-struct Coupling<float> {
-  typedef float2 type;
-  static __device__ __forceinline__ float2 make(float v) { return make_float2(v, v); }
-  static __device__ __forceinline__ void fma2(float2& acc, float2 j, float2 v) {
-    asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%0, %1};\n\t"
-        "fma.rn.f32x2 c, a, b, c;\n\tmov.b64 {%0, %1}, c;\n\t}"
-        : "+f"(acc.x), "+f"(acc.y)
-        : "f"(j.x), "f"(j.y), "f"(v.x), "f"(v.y));
+  __device__ __forceinline__ void add(const double* j, double x, double y) {
+#pragma unroll
+    for (int i = 0; i < NR; i += 2) {
+      const double2 w = *reinterpret_cast<const double2*>(j + i);
+      re[i] = fma(w.x, x, re[i]);
+      im[i] = fma(w.x, y, im[i]);
+      if (i + 1 < NR) {
+        re[i + 1] = fma(w.y, x, re[i + 1]);
+        im[i + 1] = fma(w.y, y, im[i + 1]);
+      }
+    }
   }
+  __device__ __forceinline__ double2 get(int i) const { return double2{re[i], im[i]}; }
 };
-template <typename R>
-struct alignas(16) CouplingPair {
-  typename Coupling<R>::type a, b;
+// FP32: two rows per packed multiply-add, so that a 16-byte read serves eight of them.
+template <int NR>
+struct ColumnSum<float, NR> {
+  static constexpr int NQ = (NR + 1) / 2;
+  unsigned long long re[NQ], im[NQ];  // rows 2q (low half) and 2q + 1
+  __device__ __forceinline__ ColumnSum() {
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) re[i] = im[i] = 0;
+  }
+  static __device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long j, unsigned long long v) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(j), "l"(v));
+  }
+  __device__ __forceinline__ void add(const float* j, float x, float y) {
+    unsigned long long xx, yy;
+    asm("mov.b64 %0, {%1, %1};" : "=l"(xx) : "f"(x));
+    asm("mov.b64 %0, {%1, %1};" : "=l"(yy) : "f"(y));
+#pragma unroll
+    for (int q = 0; q < NQ; q += 2) {
+      const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(j + 2 * q);
+      fma2(re[q], w.x, xx);
+      fma2(im[q], w.x, yy);
+      if (q + 1 < NQ) {
+        fma2(re[q + 1], w.y, xx);
+        fma2(im[q + 1], w.y, yy);
+      }
+    }
+  }
+  static __device__ __forceinline__ float half(unsigned long long v, int i) {
+    return __uint_as_float((unsigned)(i & 1 ? v >> 32 : v));
+  }
+  __device__ __forceinline__ float2 get(int i) const { return float2{half(re[i / 2], i), half(im[i / 2], i)}; }
 };
 
 // Barrier of `threads` threads; true when `fail` is set on any of them.
@@ -117,7 +157,6 @@ struct LargeItem {
 template <int N, typename R, bool CPLX, bool BACK, bool HALF>
 struct HalfColumn {
   typedef typename Vec2<R>::type R2;
-  typedef typename Coupling<R>::type JT;
   static constexpr int D = (N - 1) / 2;
   static constexpr int NR = (BACK ? D : D + 1) + (HALF ? 1 : 0);
   static constexpr int r0 = BACK ? (HALF ? N / 2 : N - D) : 0;
@@ -132,38 +171,24 @@ struct HalfColumn {
   }
   static __device__ __forceinline__ bool forward(int r, int b) { return 2 * r < N || (2 * r == N && 2 * b < N); }
 
-  // acc += J(b + k, b + r) v over the rows r
-  __device__ __forceinline__ void couple(const JT* jt, const JT* jti, int b, int site_k, R2 v) {
-    const int c0 = b + r0, copy = c0 & 1;
-    const JT* row = jt + (copy * N + site_k) * large_jrow(N) + c0 + copy;
-    static_for<0, (NR + 1) / 2>([&](auto ic) {
-      constexpr int i = 2 * decltype(ic)::value;
-      const CouplingPair<R> j = *reinterpret_cast<const CouplingPair<R>*>(row + i);
-      Coupling<R>::fma2(acc[i], j.a, v);
-      if constexpr (i + 1 < NR) Coupling<R>::fma2(acc[i + 1], j.b, v);
-    });
-    if constexpr (CPLX) {
-      const JT* ri = jti + (copy * N + site_k) * large_jrow(N) + c0 + copy;
-      const R2 w{-v.y, v.x};
-      static_for<0, (NR + 1) / 2>([&](auto ic) {
-        constexpr int i = 2 * decltype(ic)::value;
-        const CouplingPair<R> j = *reinterpret_cast<const CouplingPair<R>*>(ri + i);
-        // the table holds Ji(b + k, b + r) = -Ji(b + r, b + k); stored with that sign turned
-        Coupling<R>::fma2(acc[i], j.a, w);
-        if constexpr (i + 1 < NR) Coupling<R>::fma2(acc[i + 1], j.b, w);
-      });
-    }
+  // sum += J(b + k, b + r) v over the rows r
+  static __device__ __forceinline__ void couple(ColumnSum<R, NR>& sum, const R* jt, const R* jti, int b, int site_k, R2 v) {
+    constexpr int W = large_jcopies((int)sizeof(R));
+    const int c0 = b + r0, copy = -c0 & (W - 1);
+    const int at = (copy * N + site_k) * large_jrow(N, (int)sizeof(R)) + c0 + copy;
+    sum.add(jt + at, v.x, v.y);
+    // the table holds Ji(b + k, b + r) = -Ji(b + r, b + k); stored with that sign turned
+    if constexpr (CPLX) sum.add(jti + at, -v.y, v.x);
   }
 
-  __device__ __forceinline__ void compute(const LargeItem<R>& it, const LargeCoef<N, R>& cf, const JT* jt, const JT* jti,
+  __device__ __forceinline__ void compute(const LargeItem<R>& it, const LargeCoef<N, R>& cf, const R* jt, const R* jti,
                                           int b, int up, int dn) {
     const StageArgs<R>& S = it.S;
-#pragma unroll
-    for (int i = 0; i < NR; ++i) acc[i] = R2{R(0), R(0)};
+    ColumnSum<R, NR> sum;
     const R* diag = it.win + it.lane;
     const R2* pairs = reinterpret_cast<const R2*>(it.win + N * 32) + it.lane;
     // H' sigma, column entry by column entry
-    couple(jt, jti, b, b, R2{diag[b * 32], R(0)});
+    couple(sum, jt, jti, b, b, R2{diag[b * 32], R(0)});
     {
       const R2* p = pairs + b * 32;
       int site = b;
@@ -171,13 +196,13 @@ struct HalfColumn {
       for (int k = 1; k <= D; ++k, p += N * 32) {
         site = site + 1 == N ? 0 : site + 1;
         const R2 v = *p;
-        couple(jt, jti, b, site, R2{v.x, -v.y});
+        couple(sum, jt, jti, b, site, R2{v.x, -v.y});
       }
     }
     if constexpr (N % 2 == 0) {
       const bool low = 2 * b < N;
       const R2 v = pairs[((N / 2 - 1) * N + (low ? b : b - N / 2)) * 32];
-      couple(jt, jti, b, low ? b + N / 2 : b - N / 2, R2{v.x, low ? -v.y : v.y});
+      couple(sum, jt, jti, b, low ? b + N / 2 : b - N / 2, R2{v.x, low ? -v.y : v.y});
     }
     {
       int site = b;
@@ -185,9 +210,11 @@ struct HalfColumn {
 #pragma unroll 4
       for (int d = 1; d <= D; ++d, p += N * 32) {
         site = site == 0 ? N - 1 : site - 1;
-        couple(jt, jti, b, site, p[site * 32]);
+        couple(sum, jt, jti, b, site, p[site * 32]);
       }
     }
+#pragma unroll
+    for (int i = 0; i < NR; ++i) acc[i] = sum.get(i);
     // links of site b
     const R* sb = cf.site[b];
     R w_dn = R((dn >> 24) & 0xFF), w_up = R(1);
@@ -252,8 +279,8 @@ struct HalfColumn {
 // First phase: the elements of column b that other columns finish.
 template <int N, typename R, bool CPLX, bool HALF>
 __device__ __forceinline__ void large_hand_over(const LargeItem<R>& it, const LargeCoef<N, R>& cf,
-                                                const typename Coupling<R>::type* jt,
-                                                const typename Coupling<R>::type* jti, int b, int up, int dn,
+                                                const R* jt,
+                                                const R* jti, int b, int up, int dn,
                                                 typename Vec2<R>::type* ex) {
   typedef HalfColumn<N, R, CPLX, true, HALF> C;
   C c;
@@ -267,8 +294,8 @@ __device__ __forceinline__ void large_hand_over(const LargeItem<R>& it, const La
 // Second phase: the diagonal b and the pairs (b, b+d), the Horner update and the stores.
 template <int N, typename R, bool MIXED, bool CPLX, bool HALF>
 __device__ __forceinline__ void large_finish(const Inst& I, const LargeItem<R>& it, const LargeCoef<N, R>& cf,
-                                             const typename Coupling<R>::type* jt,
-                                             const typename Coupling<R>::type* jti, const double* __restrict__ cfd,
+                                             const R* jt,
+                                             const R* jti, const double* __restrict__ cfd,
                                              int b, int up, int dn, const typename Vec2<R>::type* ex,
                                              BlockRows<N, R>& rw, BlockRoot<MIXED ? N : 1>& br) {
   typedef typename Vec2<R>::type R2;
@@ -369,7 +396,6 @@ __global__ void __launch_bounds__(large_threads(N, (int)sizeof(R)), 1) heom_larg
   __shared__ Inst s_inst;
   __shared__ StageArgs<R> s_stage;
   __shared__ int s_stop;
-  typedef typename Coupling<R>::type JT;
   typedef typename Vec2<R>::type R2;
   constexpr int NN = N * N;
   constexpr int RS = (int)sizeof(R);
@@ -389,9 +415,9 @@ __global__ void __launch_bounds__(large_threads(N, (int)sizeof(R)), 1) heom_larg
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int set = wid / SW, sw = wid - set * SW;
   const bool lead = rank == 0 && threadIdx.x == 0;
-  JT* const jt = reinterpret_cast<JT*>(dsm);
-  JT* const jti = reinterpret_cast<JT*>(dsm + (CPLX ? large_jbytes(N) : 0));
-  unsigned char* const area = dsm + (CPLX ? 2 : 1) * large_jbytes(N) +
+  R* const jt = reinterpret_cast<R*>(dsm);
+  R* const jti = reinterpret_cast<R*>(dsm + (CPLX ? large_jbytes(N, RS) : 0));
+  unsigned char* const area = dsm + (CPLX ? 2 : 1) * large_jbytes(N, RS) +
                               (size_t)set * (large_stage_bytes(N, RS) + large_exch_bytes(N, RS));
   R* const stage = reinterpret_cast<R*>(area);
   R2* const ex = reinterpret_cast<R2*>(area + large_stage_bytes(N, RS)) + lane;
@@ -406,13 +432,13 @@ __global__ void __launch_bounds__(large_threads(N, (int)sizeof(R)), 1) heom_larg
       using L = CoefLayout<R>;
       const R* cf = static_cast<const R*>(I.coef);
       const double* rates = reinterpret_cast<const double*>(static_cast<const unsigned char*>(I.coef) + L::dbl_offset(N));
-      constexpr int JR = large_jrow(N);
-      for (int i = threadIdx.x; i < 2 * N * JR; i += blockDim.x) {
+      constexpr int JR = large_jrow(N, RS);
+      for (int i = threadIdx.x; i < large_jcopies(RS) * N * JR; i += blockDim.x) {
         const int copy = i / (N * JR), a = i / JR % N, c = i % JR - copy;
         const int col = c < 0 ? 0 : c % N;  // entries outside 0..2N-1 are never used, only read
-        jt[i] = Coupling<R>::make(cf[L::J(N) + a * L::JS(N) + col]);
+        jt[i] = cf[L::J(N) + a * L::JS(N) + col];
         // Ji(b + r, b + k), read from row b + k
-        if constexpr (CPLX) jti[i] = Coupling<R>::make(-cf[L::Ji(N) + a * L::JS(N) + col]);
+        if constexpr (CPLX) jti[i] = -cf[L::Ji(N) + a * L::JS(N) + col];
       }
       for (int i = threadIdx.x; i < 8 * N; i += blockDim.x) s_cf.site[i / 4][i % 4] = cf[L::site(N) + 4 * (i / 4 % N) + i % 4];
       for (int i = threadIdx.x; i < N; i += blockDim.x) {
