@@ -27,7 +27,7 @@
 // the kernel this one took the place of, 4x4 blocks of 16 nodes with two lanes
 // a node): mixed precision 70 us per stage [148], bound by issue slots, shared
 // memory and the barriers between the phases of the one block an SM holds; FP64
-// 1300 us [1800], bound by the FP64 pipe (the algorithm's multiply-adds alone
+// 1119 us [1800], bound by the FP64 pipe (the algorithm's multiply-adds alone
 // 1000 us).  16 sites, mixed: 9.2 us [21] at depth 4, 27.3 [66] at depth 5.
 // What made the difference in FP32, us per stage: y of a column read in one
 // batch (a load between two stores waits for its own round trip) and the stage's
@@ -291,6 +291,88 @@ __device__ __forceinline__ void large_hand_over(const LargeItem<R>& it, const La
   });
 }
 
+// What column c = b + d hands over to the pair (b, b+d), alone: for a block whose columns are shared out among CTAs.
+// The same terms in the same order as in HalfColumn.
+template <int N, typename R, bool CPLX>
+__device__ __forceinline__ void large_hand_over_one(const Inst& I, const LargeItem<R>& it, const LargeCoef<N, R>& cf,
+                                                    const R* jt, const R* jti, int b, int d,
+                                                    typename Vec2<R>::type* ex) {
+  typedef typename Vec2<R>::type R2;
+  constexpr int D = (N - 1) / 2, JR = large_jrow(N, (int)sizeof(R));
+  const StageArgs<R>& S = it.S;
+  const int c = b + d < N ? b + d : b + d - N, at = ((d - 1) * N + b) * 32;
+  const R2* pairs = reinterpret_cast<const R2*>(it.win + N * 32) + it.lane;
+  R re = R(0), im = R(0);
+  auto add = [&](int site, R x, R y) {
+    const R j = jt[site * JR + b];
+    re = fma(j, x, re);
+    im = fma(j, y, im);
+    if constexpr (CPLX) {
+      const R ji = jti[site * JR + b];
+      re = fma(ji, -y, re);
+      im = fma(ji, x, im);
+    }
+  };
+  add(c, it.win[c * 32 + it.lane], R(0));
+  {
+    const R2* p = pairs + c * 32;
+    int site = c;
+#pragma unroll 4
+    for (int k = 1; k <= D; ++k, p += N * 32) {
+      site = site + 1 == N ? 0 : site + 1;
+      const R2 v = *p;
+      add(site, v.x, -v.y);
+    }
+  }
+  if constexpr (N % 2 == 0) {
+    const bool low = 2 * c < N;
+    const R2 v = pairs[((N / 2 - 1) * N + (low ? c : c - N / 2)) * 32];
+    add(low ? c + N / 2 : c - N / 2, v.x, low ? -v.y : v.y);
+  }
+  {
+    int site = c;
+    const R2* p = pairs;
+#pragma unroll 4
+    for (int k = 1; k <= D; ++k, p += N * 32) {
+      site = site == 0 ? N - 1 : site - 1;
+      const R2 v = p[site * 32];
+      add(site, v.x, v.y);
+    }
+  }
+  const int up = I.up[c * I.Mpad + it.nb * 32 + it.lane], dn = I.dn[c * I.Mpad + it.nb * 32 + it.lane];
+  const R* sb = cf.site[c];
+  const R n_c = dn < 0 ? R(0) : R(dn >> 24);
+  auto linked = [&](int l) {
+    return reinterpret_cast<const R2*>(S.win + (size_t)(l >= 0 ? (unsigned)(l >> 5) : S.zero) * (N * N * 32) + N * 32);
+  };
+  if (__any_sync(0xFFFFFFFFu, dn >= 0)) {
+    const int m = dn < 0 ? -1 : (dn & 0xFFFFFF);
+    const R w = S.wsc ? scaled_dn(S.wsc, S.wstride, c, n_c) : n_c;
+    const R al = w * sb[2], be = w * sb[3];
+    const R2 v = linked(m)[(m & 31) + at];
+    re += al * v.x;
+    re -= be * v.y;
+    im += al * v.y;
+    im += be * v.x;
+  }
+  if (__any_sync(0xFFFFFFFFu, up >= 0)) {
+    const R w = S.wsc ? scaled_up(S.wsc, S.wstride, c, n_c) : R(1);
+    const R2 v = linked(up)[(up & 31) + at];
+    re += w * v.x;
+    im += w * v.y;
+  }
+  if (S.terminator) {
+    const R q = up < 0 ? (n_c + R(1)) / (it.ng + cf.gam[c]) : R(0);
+    const R ca = q * sb[2], cb = q * sb[3];
+    const R2 v = pairs[at];
+    re += cb * v.x;
+    re += ca * v.y;
+    im += cb * v.y;
+    im -= ca * v.x;
+  }
+  ex[at] = R2{im, -re};  // P = -i Q
+}
+
 // Second phase: the diagonal b and the pairs (b, b+d), the Horner update and the stores.
 template <int N, typename R, bool MIXED, bool CPLX, bool HALF>
 __device__ __forceinline__ void large_finish(const Inst& I, const LargeItem<R>& it, const LargeCoef<N, R>& cf,
@@ -400,7 +482,7 @@ __global__ void __launch_bounds__(large_threads(N, (int)sizeof(R)), 1) heom_larg
   constexpr int NN = N * N;
   constexpr int RS = (int)sizeof(R);
   constexpr int SW = large_set_warps(N, RS), SETS = large_sets(N, RS);
-  constexpr bool STAGED = RS == 4, EVEN = N % 2 == 0;
+  constexpr bool STAGED = RS == 4, EVEN = N % 2 == 0, SHARE = RS == 8;
 
   int team, rank, team_size;
   if (A.mode == 0) {
@@ -449,6 +531,13 @@ __global__ void __launch_bounds__(large_threads(N, (int)sizeof(R)), 1) heom_larg
       }
     }
     const int nblk = (I.M + 31) >> 5;
+    // FP64: rounds in which every set has a block of its own, and the parts of each block of the round after them.
+    // With fewer blocks left than sets, several sets take a share of the columns of one, and compute the elements that
+    // other columns would hand over themselves: more reads, the same arithmetic, and fewer idle sets.  The root's
+    // block is never shared.  24 sites, depth 4 (640 blocks, 152 sets): 1300 -> 1119 us per stage.  FP32, bound by issue
+    // slots, shared memory and barriers, gained 2 % there and lost 3 to 5 % where nothing is shared.
+    const int slots = SETS * team_size, full = nblk / slots;
+    const int parts = full > 0 && nblk > full * slots ? min(slots / (nblk - full * slots), N / 3) : 1;
     if (lead) {
       s_rows.os = OutStep{I.out_every == 1, 1};
       s_rows.rows.pending = -1;
@@ -500,8 +589,20 @@ __global__ void __launch_bounds__(large_threads(N, (int)sizeof(R)), 1) heom_larg
         const StageArgs<R>& S = s_stage;
         LargeItem<R> it{s_stage, nullptr, 0, lane, R(0)};
 #pragma unroll 1
-        for (int lb = set; lb * team_size + rank < nblk; lb += SETS) {
+        for (int lb = set;; lb += SETS) {
           it.nb = lb * team_size + rank;
+          int b0 = 0, b1 = N;
+          if constexpr (SHARE) {
+            if (lb >= full * SETS) {
+              // the blocks of the last round, each in `parts` parts of its columns
+              if (lb >= (full + 1) * SETS) break;
+              const int slot = set * team_size + rank, part = slot % parts;
+              it.nb = full * SETS * team_size + slot / parts;
+              b0 = part * N / parts;
+              b1 = (part + 1) * N / parts;
+            }
+          }
+          if (it.nb >= nblk) break;
           const R* src = S.win + (size_t)it.nb * (NN * 32);
           if constexpr (STAGED) {
             const int tid = sw * 32 + lane;
@@ -521,15 +622,24 @@ __global__ void __launch_bounds__(large_threads(N, (int)sizeof(R)), 1) heom_larg
             it.win = src;
           }
           it.ng = S.ngam[it.nb * 32 + lane];
+          if (!SHARE || b1 - b0 == N) {
 #pragma unroll 1
-          for (int b = sw; b < N; b += SW) {
-            const int up = I.up[b * I.Mpad + it.nb * 32 + lane], dn = I.dn[b * I.Mpad + it.nb * 32 + lane];
-            if (EVEN && 2 * b >= N) large_hand_over<N, R, CPLX, EVEN>(it, s_cf, jt, jti, b, up, dn, ex);
-            else large_hand_over<N, R, CPLX, false>(it, s_cf, jt, jti, b, up, dn, ex);
+            for (int b = sw; b < N; b += SW) {
+              const int up = I.up[b * I.Mpad + it.nb * 32 + lane], dn = I.dn[b * I.Mpad + it.nb * 32 + lane];
+              if (EVEN && 2 * b >= N) large_hand_over<N, R, CPLX, EVEN>(it, s_cf, jt, jti, b, up, dn, ex);
+              else large_hand_over<N, R, CPLX, false>(it, s_cf, jt, jti, b, up, dn, ex);
+            }
+          } else if constexpr (SHARE) {
+            constexpr int H = N / 2;
+#pragma unroll 1
+            for (int i = sw; i < (b1 - b0) * H; i += SW) {
+              const int b = b0 + i / H, d = 1 + i % H;
+              if (!EVEN || d < H || 2 * b < N) large_hand_over_one<N, R, CPLX>(I, it, s_cf, jt, jti, b, d, ex);
+            }
           }
           set_sync(1 + set, 32 * SW);
 #pragma unroll 1
-          for (int b = sw; b < N; b += SW) {
+          for (int b = b0 + sw; b < b1; b += SW) {
             const int up = I.up[b * I.Mpad + it.nb * 32 + lane], dn = I.dn[b * I.Mpad + it.nb * 32 + lane];
             if (EVEN && 2 * b < N)
               large_finish<N, R, MIXED, CPLX, EVEN>(I, it, s_cf, jt, jti, s_rates, b, up, dn, ex, s_rows, s_root);
