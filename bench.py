@@ -602,14 +602,18 @@ def main():
 
 
 def kernel_name(launch, N, prec):
-    mode = launch.get("mode") if isinstance(launch, dict) else None
+    launch = launch if isinstance(launch, dict) else {}
+    mode = launch.get("mode")
     if N > 8:
         return "heom_large_kernel<%s>" % prec
     if mode == 2:
         return "heom_smem_kernel<%d> (distributed shared memory)" % N
+    if mode == 3 and launch.get("team_ctas", 1) > (2 if N == 8 else 3):
+        return "heom_block_kernel<%d, %s> (cooperative grid)" % (N, prec)
     if mode == 3:
         return "heom_flow_kernel<%d, %s> (dataflow, %d threads per CTA)" % (N, prec, launch.get("block_threads", 0))
-    return "heom_engine_kernel<%d, %s>%s" % (N, prec, " (cooperative grid)" if mode == 1 else "")
+    name = "heom_block_kernel" if launch.get("node_threads") in (1, 2, 4) else "heom_engine_kernel"
+    return "%s<%d, %s>%s" % (name, N, prec, " (cooperative grid)" if mode == 1 else "")
 
 
 def bench_large(heom, torch, stream, peak, peak_kind, steps=0):
@@ -793,7 +797,7 @@ def bench_batched(heom, torch, stream, steps=0, filter_scan=True):
         pb.close()
         keeps = [heom.filter_select(7, w["params"]["K"], mags[i], 1e-5) for i, w in enumerate(ws)]
         # the kept auxiliaries are propagated unscaled (the same node set and rho), which runs the
-        # batch's register-view kernels
+        # batch's throughput engine
         fb = heom.Batch([w["params"] for w in ws], "fp32", stream=stream, keep=keeps)
         fb.set_rho0([w["rho0"] for w in ws])
         g0 = torch.cuda.Event(enable_timing=True)
@@ -814,8 +818,8 @@ def bench_batched(heom, torch, stream, steps=0, filter_scan=True):
     solves = len(ws) / (ms * 1e-3)
     plain = len(ws) / (plain_ms * 1e-3)
     peak, peak_kind = peaks()
-    roof = roofline_block(7, nodes, nsteps, ms, 4, peak, peak_kind, traffic_from_profile("engine_batched_scan.md"),
-                          "heom_engine_kernel<7, f32> (batched persistent launch)")
+    roof = roofline_block(7, nodes, nsteps, ms, 4, peak, peak_kind, traffic_from_profile("block_batched_scan.md"),
+                          "heom_block_kernel<7, f32> (batched persistent launch)")
     return {"workload": "256 x N=7 trap, K~U{4..8}, lambda~U(2,200), T~U(77,300), 5 ps, fp32 mixed",
             "solves_per_s": solves, "node_rhs_per_s": nodes * 4.0 * nsteps / (ms * 1e-3),
             "ms": ms, "total_nodes": nodes, "eta_mean": float(np.mean(eta)), "launch": launch, "roofline": roof,

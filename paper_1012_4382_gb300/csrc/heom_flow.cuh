@@ -609,8 +609,8 @@ __global__ void __launch_bounds__(NPT == 1 ? kFlowMaxThreads : kFlowMaxThreadsMu
 // of a pair are separate threads, terms that are zero in a whole warp are
 // skipped, and the output rows (sums and conversions in double) are left to one
 // more warp.  us per step with a row every step, two sites, depth 4, FP64: 10.2 as
-// a cluster launch of the load views, 8.4 of the throughput engine, 3.4 here
-// with the rows written by the root's warp.
+// a cluster launch of the load views, 8.4 of the throughput engine, 3.4 here;
+// seven sites, depth 3: mixed 24.5 -> 5.3, FP64 52 -> 10.3.
 template <int N, typename R, bool CPLX>
 __host__ __device__ constexpr int flow_small_terms() {
   return (flow_nre(N, CPLX) > flow_nim(N, CPLX) ? flow_nre(N, CPLX) : flow_nim(N, CPLX)) + 6;
