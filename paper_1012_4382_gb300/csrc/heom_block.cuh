@@ -26,10 +26,10 @@
 //
 // Bound and measured (us per RK4 step, whole grid, FMO-like N = 7 models; in
 // brackets the pair-by-pair kernels this engine took the place of): mixed
-// precision depth 8 13.0 [17.5], depth 10 17.8 [65], depth 12 32.9 [87]; FP64
+// precision depth 8 13.2 [17.5], depth 10 18 [65], depth 12 35.5 [92]; FP64
 // depth 8 74 [76], depth 10 143 [184].  In mixed precision a stage costs about
 // 2.4 us (grid barrier 1.2, one trip to L2 and the exchange) plus 0.52 us per
-// node block of an SM, where the SM issues about 60 % of its slots (28 warps);
+// node block of an SM, where the SM issues about half of its slots;
 // FP64 is bound by the FP64 pipe: about 980 double-precision instructions per
 // 32 nodes at 64 cycles on four sub-partitions, 8.1 us per block.  Tried and
 // dropped: the whole matrix or half of it per thread (168 registers, 12 warps:
@@ -50,9 +50,14 @@
 namespace heom {
 
 // Sets (N warps each) of the largest CTA, and the threads the kernels are
-// compiled for.
+// compiled for.  FP32: three sets at N = 7 (80 registers a thread), two at N = 8
+// (128).  With up to 28 warps (72 registers, 212 bytes of spills read back at N = 7,
+// 172 at N = 8) depth 8 took 15.3 us per step against 13.2, depth 12 37.5 against 35.5,
+// a scan of 256 hierarchies 29.6 ms against 28.6, a serving burst 46.0 ms against 41.8;
+// with 24 the burst 46.0 (three sets at N = 8), with 18 the scan 33.2.  FP64: 144
+// registers at N = 7.
 __host__ __device__ constexpr int block_max_sets(int N, int rsize) {
-  const int warps = rsize == 8 ? 16 : 28;  // at N = 7: 144 registers a thread in FP64, 72 in FP32
+  const int warps = rsize == 8 ? 16 : 21;
   return warps / N < 1 ? 1 : (warps / N > 14 ? 14 : warps / N);
 }
 __host__ __device__ constexpr int block_max_threads(int N, int rsize) { return 32 * N * block_max_sets(N, rsize); }
