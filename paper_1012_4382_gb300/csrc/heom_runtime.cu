@@ -743,7 +743,7 @@ struct Engine {
   std::vector<int*> ovr_done;
   std::vector<int64_t> ovr_every;
   DevBuf d_args, d_status, d_gsync, d_out;
-  DevBuf d_roots;  // set_rho0_all: where each instance's root goes, then the matrices
+  DevBuf d_roots;  // batches: where each instance's root goes, then the matrices (make_root_table)
   PinnedBuf h_args;
   cudaEvent_t args_done = nullptr;
   bool args_pending = false;
@@ -801,6 +801,7 @@ struct Engine {
     }
     for (auto& in : inst)
       if (!cfg.count(in->N)) cfg[in->N] = default_cfg(in->N, count);
+    if (batch) TRY(make_root_table());
     // rho(0) = |0><0| everywhere
     std::vector<double> rho;
     for (int i = 0; i < count; ++i) {
@@ -1095,6 +1096,25 @@ struct Engine {
     return set_rho0_device(i, in.stage.as<double>());
   }
 
+  // Where the matrices of a batch's rho(0) go, in device memory, with room for the matrices behind it.  Built while the
+  // batch is made, so that set_rho0_all needs no allocation and never meets a table that was not filled.
+  int make_root_table() {
+    const int count = (int)inst.size();
+    std::vector<RootTarget> t(count);
+    size_t total = 0;
+    for (int i = 0; i < count; ++i) {
+      Instance& in = *inst[i];
+      t[i] = RootTarget{in.y.p, root_ptr(in, 0), in.acc.as<double>(), (int64_t)heom::state_reals(in.N, in.Mpad),
+                        (int64_t)total, in.N, prec == HEOM_FP64};
+      total += 2 * (size_t)in.N * in.N;
+    }
+    TRY(d_roots.alloc(root_table_bytes() + sizeof(double) * total, hooks));
+    CUDA_TRY(cudaMemcpyAsync(d_roots.p, t.data(), sizeof(RootTarget) * count, cudaMemcpyHostToDevice, stream));
+    CUDA_TRY(cudaStreamSynchronize(stream));
+    return HEOM_OK;
+  }
+  size_t root_table_bytes() const { return (sizeof(RootTarget) * inst.size() + 15) / 16 * 16; }
+
   // rho(0) of every instance (concatenated N*N complex matrices): one copy and one launch for up to 65535 instances,
   // where a copy, a clear, a launch and a wait per instance took 35 us each (256 instances: 9 ms of a 33 ms scan of 60
   // steps).  Blocking.
@@ -1105,21 +1125,7 @@ struct Engine {
       TRY(validate_rho(rho_all + total, inst[i]->N));
       total += 2 * (size_t)inst[i]->N * inst[i]->N;
     }
-    const size_t tbytes = (sizeof(RootTarget) * count + 15) / 16 * 16;
-    if (!d_roots.p) {
-      std::vector<RootTarget> t(count);
-      size_t off = 0;
-      for (int i = 0; i < count; ++i) {
-        Instance& in = *inst[i];
-        t[i] = RootTarget{in.y.p, root_ptr(in, 0), in.acc.as<double>(), (int64_t)heom::state_reals(in.N, in.Mpad),
-                          (int64_t)off, in.N, prec == HEOM_FP64};
-        off += 2 * (size_t)in.N * in.N;
-      }
-      TRY(d_roots.alloc(tbytes + sizeof(double) * total, hooks));
-      CUDA_TRY(cudaMemcpyAsync(d_roots.p, t.data(), sizeof(RootTarget) * count, cudaMemcpyHostToDevice, stream));
-      CUDA_TRY(cudaStreamSynchronize(stream));
-    }
-    double* d_rho = reinterpret_cast<double*>(d_roots.as<unsigned char>() + tbytes);
+    double* d_rho = reinterpret_cast<double*>(d_roots.as<unsigned char>() + root_table_bytes());
     CUDA_TRY(cudaMemcpyAsync(d_rho, rho_all, sizeof(double) * total, cudaMemcpyHostToDevice, stream));
     for (int i = 0; i < count; i += 65535)
       set_roots_kernel<<<dim3(8, std::min(count - i, 65535)), 256, 0, stream>>>(d_roots.as<RootTarget>() + i, d_rho);
