@@ -160,6 +160,20 @@ struct PinnedBuf {
   }
 };
 
+// Lets kernel k be launched with all the dynamic shared memory the current device has beside the kernel's static
+// part.  The limit is one per kernel and process, so every launch sets it to the same value: with each launch's own size,
+// threads that launch one kernel for hierarchies of different sizes lowered it under each other (launches refused, and
+// shapes reported as not resident).
+int raise_smem_limit(const void* k) {
+  int device = 0, optin = 0;
+  CUDA_TRY(cudaGetDevice(&device));
+  CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
+  cudaFuncAttributes at;
+  CUDA_TRY(cudaFuncGetAttributes(&at, k));
+  CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)at.sharedSizeBytes));
+  return HEOM_OK;
+}
+
 // ------------------------------------------------------------- utilities
 
 // The root node of the mixed path is kept in float-float (hi, lo) pairs.
@@ -902,7 +916,7 @@ struct Engine {
           if (S < 1 || !k) continue;
           const int dyn = heom::flow_smem_bytes(N, S * npt, (int)rsize());
           int per_sm = 0;
-          if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn) == cudaSuccess &&
+          if (raise_smem_limit(k) == HEOM_OK &&
               cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, S * U, dyn) == cudaSuccess &&
               (int64_t)per_sm * sms >= (Mmax + S * npt - 1) / (S * npt)) {
             c.mode = 3;
@@ -1403,7 +1417,7 @@ struct Engine {
     const int SL = S * npt;  // nodes of a CTA's slice
     const int grid = (int)((in.M + SL - 1) / SL);
     const int dyn = heom::flow_smem_bytes(N, SL, (int)rsize());
-    CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+    TRY(raise_smem_limit(k));
     int per_sm = 0;
     CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, dyn));
     if ((int64_t)per_sm * sms < grid)
@@ -1529,7 +1543,7 @@ struct Engine {
       return 0;
     }
     if (c.team_ctas > 8) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    if (dyn > 0) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+    if (dyn > 0 && raise_smem_limit(k) != HEOM_OK) return 0;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(c.team_ctas);
     lc.blockDim = dim3(cta_threads(N, sc, c));
@@ -1563,7 +1577,7 @@ struct Engine {
     const int block = cta_threads(N, sc, c);
     if (c.mode == 1) {
       int per_sm = 0;
-      if (dyn > 0) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+      if (dyn > 0) TRY(raise_smem_limit(k));
       CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, dyn));
       if (per_sm < 1) return fail(HEOM_ECUDA, "block of %d threads cannot be resident", block);
       const int grid = per_sm * sms;
@@ -1573,7 +1587,7 @@ struct Engine {
       return HEOM_OK;
     }
     if (c.team_ctas > 8) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-    if (dyn > 0) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+    if (dyn > 0) TRY(raise_smem_limit(k));
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(nteams * c.team_ctas);
     lc.blockDim = dim3(block);
@@ -2572,7 +2586,7 @@ extern "C" int heom_propagate_static(const heom_params* params, const double* d_
   const int threads = 32 * N * sets;
   const int dyn = heom::block_exch_bytes(N, (int)rs, sets);
   int link_cache = 0;
-  if (dyn > 0) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn));
+  if (dyn > 0) TRY(raise_smem_limit(k));
   cudaLaunchConfig_t lc = {};
   cudaLaunchAttribute at[1];
   for (;;) {
