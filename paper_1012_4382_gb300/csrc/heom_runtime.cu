@@ -1980,22 +1980,23 @@ int heom_ctx_num_nodes(const heom_ctx* ctx, int64_t* out) {
 int heom_set_launch(heom_ctx* ctx, int32_t mode, int32_t team_ctas, int32_t block_threads, int32_t node_threads) {
   if (!ctx) return fail(HEOM_EINVAL, "ctx is NULL");
   LaunchCfg& c = ctx->e.cfg[ctx->e.inst[0]->N];
+  LaunchCfg n = c;
   if (c.automatic && mode < 0 && (team_ctas > 0 || block_threads > 0 || node_threads > 0)) {
     // team_ctas, block_threads or node_threads alone, on a small hierarchy whose shape was never set: they are those of
     // a cluster launch, as they mean nothing to the one-CTA kernel the default runs
-    c.mode = 0;
-    c.team_ctas = 1;
-    c.block = ctx->e.max_block();
-    c.G = ctx->e.inst[0]->scaled ? 4 : 2;
+    n.mode = 0;
+    n.team_ctas = 1;
+    n.block = ctx->e.max_block();
+    n.G = ctx->e.inst[0]->scaled ? 4 : 2;
   }
-  LaunchCfg n = c;
+  const int from = n.mode;
   n.automatic = false;
   if (mode >= 0) n.mode = mode;
   if (team_ctas > 0) n.team_ctas = team_ctas;
   if (block_threads > 0) n.block = block_threads;
   if (node_threads > 0) n.G = node_threads;
   if (n.mode < 0 || n.mode > 3) return fail(HEOM_EINVAL, "mode must be 0, 1, 2 or 3");
-  if ((n.mode == 3) != (c.mode == 3)) {
+  if ((n.mode == 3) != (from == 3)) {
     // a block size or team size (nodes per thread in mode 3) of the other family of
     // engines does not carry over: take that family's default
     const int N = ctx->e.inst[0]->N;
