@@ -292,7 +292,9 @@ int heom_ctx_num_nodes(const heom_ctx* ctx, int64_t* out);
  * one node per thread: 12 nodes in 336 threads); a call whose CTAs cannot all
  * be resident fails with HEOM_EINVAL.  Switching between mode 3 and the
  * other modes without giving team_ctas or block_threads resets them to that
- * family's default.  node_threads: threads sharing one node's matrix, 1..32;
+ * family's default, and a hierarchy of less than 256 nodes whose shape was never
+ * set takes what a call leaves out from a cluster of about 32 nodes per CTA (128 in
+ * mode 2).  node_threads: threads sharing one node's matrix, 1..32;
  * 1, 2 and 4 select, in modes 0 and 1 with N <= 8, the throughput engine, which
  * gives a node N threads and a CTA about twice block_threads threads whatever
  * the count (scaled hierarchies: 4 only); not used by mode 3.  A

@@ -946,6 +946,31 @@ struct Engine {
     return c;
   }
 
+  // What heom_set_launch starts from on a small hierarchy (N <= 8) whose shape was never set, for the values that the
+  // call leaves out: they are those of a cluster launch, as they mean nothing to the one-CTA and dataflow kernels the
+  // default runs.  The throughput engine with about one block of 32 nodes per CTA.  Shared memory with 128 nodes per CTA
+  // for mode 2, and in mixed precision for node_threads alone that select the load views, which it holds faster: 4 sites
+  // depth 4, node_threads 8, 11.7 us a step against 15.0 in device memory, 5 sites depth 5 15.8 against 21.  With one CTA
+  // for all of them, 7 sites depth 3 in FP64 took 134 us a step (now 40), 5 sites depth 5 113 (20).
+  LaunchCfg cluster_cfg(const Instance& in, int mode, int node_threads) const {
+    LaunchCfg c;
+    const bool views = node_threads > 0 && node_threads != 1 && node_threads != 2 && node_threads != 4;
+    if (mode == 2 || (mode < 0 && views && prec == HEOM_FP32_MIXED && !in.scaled)) {
+      c.mode = 2;
+      c.block = 512;
+      c.G = 4;
+      while (c.team_ctas < 16 && (c.team_ctas * 128 < in.M ||
+                                  heom::smem_dyn_bytes(in.N, smem_slice(in.M, c.team_ctas)) > max_dyn_smem()))
+        c.team_ctas <<= 1;
+      return c;
+    }
+    c.mode = mode < 0 ? 0 : mode;
+    c.block = max_block();
+    c.G = in.scaled ? 4 : 2;
+    while (c.team_ctas < 16 && c.team_ctas * 32 < in.M) c.team_ctas <<= 1;
+    return c;
+  }
+
   int add_instance(const heom_params& p) {
     auto in = std::make_unique<Instance>();
     in->N = p.N;
@@ -1981,14 +2006,8 @@ int heom_set_launch(heom_ctx* ctx, int32_t mode, int32_t team_ctas, int32_t bloc
   if (!ctx) return fail(HEOM_EINVAL, "ctx is NULL");
   LaunchCfg& c = ctx->e.cfg[ctx->e.inst[0]->N];
   LaunchCfg n = c;
-  if (c.automatic && mode < 0 && (team_ctas > 0 || block_threads > 0 || node_threads > 0)) {
-    // team_ctas, block_threads or node_threads alone, on a small hierarchy whose shape was never set: they are those of
-    // a cluster launch, as they mean nothing to the one-CTA kernel the default runs
-    n.mode = 0;
-    n.team_ctas = 1;
-    n.block = ctx->e.max_block();
-    n.G = ctx->e.inst[0]->scaled ? 4 : 2;
-  }
+  if (c.automatic && (mode < 0 ? team_ctas > 0 || block_threads > 0 || node_threads > 0 : mode < 3))
+    n = ctx->e.cluster_cfg(*ctx->e.inst[0], mode, node_threads);
   const int from = n.mode;
   n.automatic = false;
   if (mode >= 0) n.mode = mode;

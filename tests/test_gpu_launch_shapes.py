@@ -1,6 +1,8 @@
 """heom_set_launch on a small hierarchy that still has its default shape."""
+import numpy as np
 import pytest
 
+import oracle
 from paper_1012_4382_gb300 import build as heom_build
 from paper_1012_4382_gb300 import heom, workloads
 
@@ -26,3 +28,20 @@ def test_refused_shape_leaves_the_default(bad, precision):
         assert c.get_launch() == shape
         c.set_launch(node_threads=8)  # and the context still counts as one whose shape was never set
         assert c.get_launch()["mode"] != 3
+
+
+# 5 sites, depth 5: 252 nodes, eight blocks of 32
+@pytest.mark.parametrize("precision,call,mode,team", [
+    ("fp64", dict(mode=0), 0, 8), ("fp64", dict(block_threads=128), 0, 8), ("fp64", dict(node_threads=8), 0, 8),
+    ("fp64", dict(team_ctas=2), 0, 2), ("fp32", dict(mode=0), 0, 8), ("fp32", dict(mode=2), 2, 2),
+    ("fp32", dict(node_threads=8), 2, 2), ("fp32", dict(node_threads=4), 0, 8)])
+def test_values_left_out_are_those_of_a_cluster_launch(precision, call, mode, team):
+    w = workloads.random_instance(5, 5, seed=12)
+    o = oracle.propagate(w["params"], w["rho0"], 1.0, 20, 5)
+    tol = 1e-10 if precision == "fp64" else 1e-5
+    with heom.Context(w["params"], precision) as c:
+        c.set_launch(**call)
+        shape = c.get_launch()
+        assert (shape["mode"], shape["team_ctas"]) == (mode, team)
+        c.set_rho0(w["rho0"])
+        assert np.abs(c.propagate(1.0, 20, 5)["pops"] - o["pops"]).max() < tol
