@@ -948,10 +948,10 @@ struct Engine {
 
   // What heom_set_launch starts from on a small hierarchy (N <= 8) whose shape was never set, for the values that the
   // call leaves out: they are those of a cluster launch, as they mean nothing to the one-CTA and dataflow kernels the
-  // default runs.  The throughput engine with about one block of 32 nodes per CTA.  Shared memory with 128 nodes per CTA
-  // for mode 2, and in mixed precision for node_threads alone that select the load views, which it holds faster: 4 sites
-  // depth 4, node_threads 8, 11.7 us a step against 15.0 in device memory, 5 sites depth 5 15.8 against 21.  With one CTA
-  // for all of them, 7 sites depth 3 in FP64 took 134 us a step (now 40), 5 sites depth 5 113 (20).
+  // default runs.  The throughput engine with about one block of 32 nodes per CTA (FP64, one CTA in brackets: 7 sites
+  // depth 3 40 us a step [134], 5 sites depth 5 20 [113]).  Shared memory with 128 nodes per CTA for mode 2, and in
+  // mixed precision for node_threads alone that select the load views, which run faster from it: 4 sites depth 4,
+  // node_threads 8, 12.2 us a step against 15.6 in device memory.
   LaunchCfg cluster_cfg(const Instance& in, int mode, int node_threads) const {
     LaunchCfg c;
     const bool views = node_threads > 0 && node_threads != 1 && node_threads != 2 && node_threads != 4;
@@ -967,6 +967,9 @@ struct Engine {
     c.mode = mode < 0 ? 0 : mode;
     c.block = max_block();
     c.G = in.scaled ? 4 : 2;
+    // one CTA where its sets take all blocks at once and the FP64 pipe does not bind (mixed, 4 sites depth 4: 4.9 us a step
+    // against 6.4 in a cluster; seven sites depth 3, four blocks on three sets: 13.1 against 9.4)
+    if (prec == HEOM_FP32_MIXED && in.M <= 32 * heom::block_sets(in.N, (int)rsize(), c.block)) return c;
     while (c.team_ctas < 16 && c.team_ctas * 32 < in.M) c.team_ctas <<= 1;
     return c;
   }

@@ -45,3 +45,13 @@ def test_values_left_out_are_those_of_a_cluster_launch(precision, call, mode, te
         assert (shape["mode"], shape["team_ctas"]) == (mode, team)
         c.set_rho0(w["rho0"])
         assert np.abs(c.propagate(1.0, 20, 5)["pops"] - o["pops"]).max() < tol
+
+
+def test_mixed_hierarchy_that_one_cta_takes_at_once_stays_in_one():
+    w = workloads.random_instance(4, 4, seed=13)  # 70 nodes, three blocks of 32 on the five sets of a CTA
+    o = oracle.propagate(w["params"], w["rho0"], 1.0, 20, 5)
+    with heom.Context(w["params"], "fp32") as c:
+        c.set_launch(node_threads=4)
+        assert c.get_launch()["team_ctas"] == 1
+        c.set_rho0(w["rho0"])
+        assert np.abs(c.propagate(1.0, 20, 5)["pops"] - o["pops"]).max() < 1e-5
