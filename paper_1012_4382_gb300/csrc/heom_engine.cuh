@@ -1563,7 +1563,10 @@ __global__ void __launch_bounds__(512) heom_smem_kernel(EngineArgs A, int B) {
     float* gyw = static_cast<float*>(I.y);
     for (int idx = threadIdx.x; idx < NN * B; idx += blockDim.x) {
       const int p = idx / B, l = idx - (idx / B) * B;
-      if (l < nloc) gyw[node_col<N>(n0 + l) + p * 32] = sy[idx];
+      // the blocked index from the element-major one: with node_col<N>(n0 + l) + 32 p the compiler gives the step loop
+      // fewer registers (three sites, register view, 94 instead of 110: depth 24 on 8 CTAs 21.2 us a step against 17.3)
+      const int o = p * Mp + n0 + l, q = o / I.Mpad;
+      if (l < nloc) gyw[node_col<N>(o - q * I.Mpad) + q * 32] = sy[idx];
     }
     cluster_sync_all();  // no CTA reuses or leaves its slice while others may still read it
     if (lead) signal_done(I);

@@ -45,3 +45,25 @@ def test_dataflow_kernels_spill_no_more_than_with_an_element_major_state(tmp_pat
         assert seen[k][0] <= st and seen[k][1] <= ld, (k, seen[k])
         if (real,) + k in FULL_BUDGET:
             assert seen[k][2] > 84, (k, seen[k])
+
+
+def test_shared_memory_kernels_keep_their_registers(tmp_path):
+    """The kernels of launch mode 2, three and six sites: what the compiler gave their step loops before the state was
+    blocked; fewer went with longer steps (the loads of a stage are issued in smaller groups)."""
+    src = tmp_path / "smem.cu"
+    want = {(3, True): 110, (6, True): 128}
+    src.write_text('#include "heom_engine.cuh"\nnamespace heom { const void* kernels[] = {%s}; }\n' % ", ".join(
+        "(const void*)heom_smem_kernel<%d, false, %s>" % (N, str(reg).lower()) for N, reg in want))
+    r = subprocess.run([heom_build._nvcc()] + heom_build.ARCH + ["-O3", "-std=c++17", "-I" + heom_build.INCLUDE,
+                       "-I" + heom_build.CSRC, "-Xptxas", "-v", "-c", str(src), "-o", str(tmp_path / "smem.o")],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    key, seen = None, {}
+    for line in r.stderr.splitlines():
+        m = re.search(r"heom_smem_kernelILi(\d)ELb0ELb([01])E", line)
+        if m:
+            key = (int(m.group(1)), m.group(2) == "1")
+        m = re.search(r"Used (\d+) registers", line)
+        if m:
+            seen[key] = int(m.group(1))
+    assert seen == want
