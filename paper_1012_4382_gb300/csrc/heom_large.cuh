@@ -69,6 +69,22 @@ __host__ __device__ constexpr int large_smem_bytes(int N, int rsize, bool cplx) 
          large_sets(N, rsize) * (large_stage_bytes(N, rsize) + large_exch_bytes(N, rsize));
 }
 
+// Parts in which a team of `team` CTAs with `sets` sets each computes its last `rest` < sets * team blocks: the fewest
+// that make the CTA with the most parts' share of a block smallest (a CTA's sets share its FP64 pipe, so a second busy
+// set gains nothing by itself: 16 sites depth 4, 152 blocks on 152 CTAs, in halves 407 us a step against 370), a smaller
+// share by less than 5 % not counted; at least three columns a part.
+__host__ __device__ constexpr int large_parts(int N, int sets, int team, int rest) {
+  int best = 1, most = rest > 0 ? (rest + team - 1) / team : 1;  // parts, and those of the fullest CTA
+  for (int p = 2; p <= N / 3 && p * rest <= sets * team; ++p) {
+    const int m = (rest * p + team - 1) / team;
+    if (20 * m * best < 19 * most * p) {
+      best = p;
+      most = m;
+    }
+  }
+  return best;
+}
+
 // The sum over k of J(k, row) sigma_k for NR rows: j holds NR couplings (and
 // what fills the last 16-byte word), x and y multiply them into the real and
 // imaginary sums.
@@ -531,23 +547,29 @@ __global__ void __launch_bounds__(large_threads(N, (int)sizeof(R)), 1) heom_larg
       }
     }
     const int nblk = (I.M + 31) >> 5;
-    // FP64: rounds in which every set has a block of its own, and the parts of each block of the round after them.
-    // With fewer blocks left than sets, several sets take a share of the columns of one, and compute the elements that
-    // other columns would hand over themselves: more reads, the same arithmetic, and fewer idle sets.  The root's
-    // block is never shared.  24 sites, depth 4 (640 blocks, 152 sets): 1300 -> 1119 us per stage.  FP32, bound by issue
-    // slots, shared memory and barriers, gained 2 % there and lost 3 to 5 % where nothing is shared.
-    const int slots = SETS * team_size, full = nblk / slots;
-    const int parts = full > 0 && nblk > full * slots ? min(slots / (nblk - full * slots), N / 3) : 1;
-    if (lead) {
+    // FP64: rounds in which every set has a block of its own, and the parts of each block of the round after them (the
+    // only one of a small hierarchy).  With fewer blocks left than sets, several sets take a share of the columns of one,
+    // and compute the elements that other columns would hand over themselves: more reads, the same arithmetic, and
+    // fewer idle CTAs (see large_parts).  24 sites, depth 4 (640 blocks, 152 CTAs): 1300 -> 1119 us per stage; depth 1 (one
+    // block, 8 CTAs): 273 -> 49.  FP32, bound by issue slots, shared memory and barriers, gained 2 % on the former and
+    // lost 3 to 5 % where nothing is shared.
+    const int slots = SETS * team_size, full = nblk / slots, rest = nblk - full * slots;
+    const int parts = SHARE ? large_parts(N, SETS, team_size, rest) : 1;
+    // the columns of the root's block this set runs: they keep its output rows and sums
+    const int slot0 = set * team_size + rank;
+    const bool root_shared = SHARE && full == 0;
+    const int rc0 = root_shared ? min(slot0, parts) * N / parts : 0;
+    const int rc1 = root_shared ? min(slot0 + 1, parts) * N / parts : (slot0 == 0 ? N : 0);
+    if (threadIdx.x == 0) {
       s_rows.os = OutStep{I.out_every == 1, 1};
       s_rows.rows.pending = -1;
       s_rows.rows.acc0 = I.acc[0];
       s_rows.rows.acc1 = I.acc[1];
+      for (int k = 0; k < N; ++k) s_rows.ea[k] = EtaAcc<R>{};
+    }
+    if (lead) {
       write_row0<N, R, MIXED>(I);
-      for (int k = 0; k < N; ++k) {  // zero the running sums of every site
-        s_rows.ea[k] = EtaAcc<R>{};
-        s_rows.ea[k].store(I, k);
-      }
+      for (int k = 0; k < N; ++k) s_rows.ea[k].store(I, k);  // zero the running sums of every site
     }
     if constexpr (MIXED) {
       for (int p = threadIdx.x; p < NN; p += blockDim.x) {
@@ -596,8 +618,8 @@ __global__ void __launch_bounds__(large_threads(N, (int)sizeof(R)), 1) heom_larg
             if (lb >= full * SETS) {
               // the blocks of the last round, each in `parts` parts of its columns
               if (lb >= (full + 1) * SETS) break;
-              const int slot = set * team_size + rank, part = slot % parts;
-              it.nb = full * SETS * team_size + slot / parts;
+              const int part = slot0 % parts;
+              it.nb = full * slots + slot0 / parts;
               b0 = part * N / parts;
               b1 = (part + 1) * N / parts;
             }
@@ -648,18 +670,18 @@ __global__ void __launch_bounds__(large_threads(N, (int)sizeof(R)), 1) heom_larg
           }
           set_sync(1 + set, 32 * SW);  // the set's areas are free again
         }
-        // lane 0 of the warps of rank 0, set 0 (which run the root's block) keep the sums of their columns
-        if (s == 3 && rank == 0 && set == 0 && lane == 0 && (s_rows.os.now || t + 1 == I.nsteps))
-          for (int b = sw; b < N; b += SW) s_rows.ea[b].store(I, b);
+        // lane 0 of the warps that run the root's block keep the sums of their columns
+        if (s == 3 && lane == 0 && (s_rows.os.now || t + 1 == I.nsteps))
+          for (int b = rc0 + sw; b < rc1; b += SW) s_rows.ea[b].store(I, b);
         if (!team_barrier(A, epoch)) return;
       }
-      if (lead) {
+      if (threadIdx.x == 0) {
         if (s_rows.os.now) s_rows.rows.pending = s_rows.os.row++;
         s_rows.os.now = t + 2 == I.out_every * s_rows.os.row;
       }
       if (I.stop_trace > 0.0 && t + 1 < I.nsteps && stop_now<R, MIXED>(I, N, &s_stop)) {
-        if (rank == 0 && set == 0 && lane == 0)
-          for (int b = sw; b < N; b += SW) s_rows.ea[b].store(I, b);
+        if (lane == 0)
+          for (int b = rc0 + sw; b < rc1; b += SW) s_rows.ea[b].store(I, b);
         done = t + 1;
         if (!team_barrier(A, epoch)) return;
         break;
