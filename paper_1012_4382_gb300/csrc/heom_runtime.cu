@@ -934,6 +934,18 @@ struct Engine {
       c.team_ctas = 1;
       c.block = max_block();
       c.G = 2;
+      // ... but eight sites in FP64 with complex H and little more than one block of 32 nodes per SM, which the throughput
+      // engine takes two rounds for: the load views in eight groups give each of the 12 warps of an SM at most one item up
+      // to 1.5 blocks per SM.  us a step, 160 to 202 blocks on 152 SMs 141 against 154 (230 blocks 184 against 155; seven
+      // sites 104 against 105).  Not with the terminator or scaled, which cost the load views more, nor with real H: 101
+      // against 105, but 117 against 113 with a row every step.
+      const int64_t nb = (Mmax + 31) / 32;
+      bool plain = true;
+      for (auto& in : inst) plain &= in->N != N || (in->complex_h && !in->terminator && !in->scaled);
+      if (prec == HEOM_FP64 && N == 8 && plain && nb > sms && 2 * nb <= 3 * sms) {
+        c.block = 128;
+        c.G = 8;
+      }
     } else {
       // many hierarchies: the throughput engine with the team size batch_team picks.  Keeping small hierarchies in
       // shared memory (mode 2) loses to it: 64 hierarchies of 70 nodes (N = 4) 14.9 us a step against 7.2, 300 of 252

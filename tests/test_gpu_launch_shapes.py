@@ -55,3 +55,28 @@ def test_mixed_hierarchy_that_one_cta_takes_at_once_stays_in_one():
         assert c.get_launch()["team_ctas"] == 1
         c.set_rho0(w["rho0"])
         assert np.abs(c.propagate(1.0, 20, 5)["pops"] - o["pops"]).max() < 1e-5
+
+
+@pytest.mark.parametrize("complex_h,terminator,keep_blocks,node_threads", [
+    (True, 0, None, 8), (False, 0, None, 2), (True, 1, None, 2), (True, 0, 152, 2), (True, 0, 153, 8),
+    (True, 0, 228, 8), (True, 0, 229, 2)])
+def test_eight_sites_fp64_just_above_one_block_per_sm(complex_h, terminator, keep_blocks, node_threads):
+    """Depth 7 (6435 nodes, 202 blocks of 32 on 152 SMs) and first nodes of depth 8, at the edges of the range in
+    which the load views are the default."""
+    K = 7 if keep_blocks is None else 8
+    w = workloads.random_instance(8, K, seed=21, complex_h=complex_h, terminator=terminator)
+    M, p, keep = heom.num_nodes(8, K), w["params"], None
+    if keep_blocks is not None:
+        keep = (np.arange(M) < 32 * keep_blocks - 5).astype(np.uint8)
+        multi, _, _ = heom.build_index(8, K)
+        pos = {tuple(m): i for i, m in enumerate(oracle.multi_indices(8, K).tolist())}
+        okeep = np.zeros(M, np.uint8)
+        okeep[[pos[tuple(m)] for m in multi[keep > 0].tolist()]] = 1
+        p = dict(p, keep=okeep)
+    o = oracle.propagate(p, w["rho0"], 1.0, 4, 2)
+    with heom.Context(w["params"], "fp64", keep=keep) as c:
+        assert c.get_launch()["mode"] == 1 and c.get_launch()["node_threads"] == node_threads
+        c.set_rho0(w["rho0"])
+        r = c.propagate(1.0, 4, 2)
+    assert np.abs(r["pops"] - o["pops"]).max() < 1e-10
+    assert np.abs(r["eta"] - o["eta"]).max() < 1e-10
