@@ -29,6 +29,7 @@
 #include "heom_flow.cuh"
 #include "heom_large.cuh"
 #include "heom_internal.h"
+#include "heom_team.h"
 
 using heom::CoefLayout;
 using heom::EngineArgs;
@@ -842,37 +843,35 @@ struct Engine {
     return c;
   }
 
-  // CTAs per team for a batch's instances with N sites: of 1, 2, 4, 8 and 16 the one whose longest-first packing of
-  // the instances onto the teams the GPU holds at once has the shortest makespan, with a stage of b node blocks per
-  // CTA taking a + m b.  Measured (us, N = 7): a = 1.5; m = 0.52 in mixed precision, 8.1 in FP64 (the FP64 pipe);
-  // m scales about as N^2.5 (N = 5: 0.25 and 3.5, N = 8: 0.73 and 12).  Per step, team sizes 1, 2, 4, 8, 16: 256 mixed
-  // instances of depth 4 to 8 543, 398, 408, 411 us (2 picked); 24 FP64 ones of depth 4 to 7 -, 1745, 884, 463, 366
-  // (16 picked; 1745 with the former fixed 2); 30 mixed of depth 7 231, 121, 64, 73, 108 (4 picked).
+  // CTAs per team for a batch's instances with N sites: the size pick_team finds among those whose teams can be resident.
+  // m, measured for N = 7 (us): 0.52 in mixed precision, 8.1 in FP64 (the FP64 pipe); it scales about as N^2.5 (N = 5:
+  // 0.25 and 3.5, N = 8: 0.73 and 12).  us per step for team sizes 1, 2, 4, 8, 16: 256 mixed instances of depth 4 to 8
+  // 543, 398, 408, 411 (2 picked); 24 FP64 ones of depth 3 to 6 1755, 889, 469, 240, 305 (8 picked); 30 mixed of depth 7
+  // 231, 121, 64, 73, 108 (4 picked).
   int batch_team(int N) const {
     std::vector<int64_t> blocks;
+    int64_t Mmax = 0;
+    int cplx = 0, sc = 0;
     for (auto& in : inst)
-      if (in->N == N) blocks.push_back((in->M + 31) / 32);
-    std::sort(blocks.begin(), blocks.end(), std::greater<int64_t>());
-    const double m = (prec == HEOM_FP64 ? 8.1 : 0.52) * std::pow(N / 7.0, 2.5);
-    int best = 1;
-    double best_t = 0.0;
-    for (int c = 1; c <= 16; c *= 2) {
-      const size_t teams = std::min<size_t>(blocks.size(), std::max(1, sms / c));
-      std::priority_queue<double, std::vector<double>, std::greater<double>> load;
-      for (size_t t = 0; t < teams; ++t) load.push(0.0);
-      double span = 0.0;
-      for (int64_t b : blocks) {
-        const double t = load.top() + 1.5 + m * (double)((b + c - 1) / c);
-        load.pop();
-        load.push(t);
-        span = std::max(span, t);
+      if (in->N == N) {
+        blocks.push_back((in->M + 31) / 32);
+        Mmax = std::max<int64_t>(Mmax, in->M);
+        cplx |= in->complex_h;
+        sc |= in->scaled;
       }
-      if (c == 1 || span < 0.98 * best_t) {
-        best = c;
-        best_t = span;
-      }
+    int resident[5];
+    for (int i = 0; i < 5; ++i) {
+      resident[i] = sms / heom::kTeamSizes[i];
+      if (!batch) continue;  // (a server gives its launches a shape of their own)
+      LaunchCfg c;
+      c.mode = 0;
+      c.team_ctas = heom::kTeamSizes[i];
+      c.block = max_block();
+      c.G = sc ? 4 : 2;
+      resident[i] = max_active_teams(N, cplx, sc, c, block_dyn(N, c, Mmax));
     }
-    return best;
+    if (batch) t_err.clear();  // sizes that cannot be resident are no error
+    return heom::pick_team(std::move(blocks), (prec == HEOM_FP64 ? 8.1 : 0.52) * std::pow(N / 7.0, 2.5), resident);
   }
 
   LaunchCfg default_cfg_plain(int N, int count) const {
@@ -1575,14 +1574,21 @@ struct Engine {
   }
 
   // Teams of this shape that fit on the GPU at once; 0 on error (message set).
-  int max_active_teams(int N, int cplx, int sc, const LaunchCfg& c, int dyn = 0) {
+  int max_active_teams(int N, int cplx, int sc, const LaunchCfg& c, int dyn = 0) const {
     const void* k = kernel_for(N, cplx, sc, c);
     if (!k) {
       fail(HEOM_EUNSUPPORTED, "no engine kernel for N=%d, launch mode %d, node_threads %d%s", N, c.mode, c.G,
            no_kernel_reason(N, sc));
       return 0;
     }
-    if (c.team_ctas > 8) CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    if (c.team_ctas > 8) {
+      const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) {
+        cudaGetLastError();
+        fail(HEOM_ECUDA, "clusters of %d CTAs: %s", c.team_ctas, cudaGetErrorString(e));
+        return 0;
+      }
+    }
     if (dyn > 0 && raise_smem_limit(k) != HEOM_OK) return 0;
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(c.team_ctas);
