@@ -166,12 +166,21 @@ struct PinnedBuf {
 // threads that launch one kernel for hierarchies of different sizes lowered it under each other (launches refused, and
 // shapes reported as not resident).
 int raise_smem_limit(const void* k) {
-  int device = 0, optin = 0;
+  // the calling thread's last kernel and its limit (a constant of kernel and device), which spares most calls two queries
+  static thread_local const void* last = nullptr;
+  static thread_local int last_device = -1, limit = 0;
+  int device = 0;
   CUDA_TRY(cudaGetDevice(&device));
-  CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
-  cudaFuncAttributes at;
-  CUDA_TRY(cudaFuncGetAttributes(&at, k));
-  CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)at.sharedSizeBytes));
+  if (k != last || device != last_device) {
+    int optin = 0;
+    cudaFuncAttributes at;
+    CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
+    CUDA_TRY(cudaFuncGetAttributes(&at, k));
+    limit = optin - (int)at.sharedSizeBytes;
+    last = k;
+    last_device = device;
+  }
+  CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, limit));
   return HEOM_OK;
 }
 
