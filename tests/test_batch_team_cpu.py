@@ -54,6 +54,15 @@ def test_packing_counts_the_teams_that_exist(pick):
     assert pick(8.1, IDEAL, blocks) == 16
 
 
+def test_small_hierarchies_stay_in_one_cta(pick):
+    # mixed precision; m as for three, four and seven sites (us per step with one CTA and the best cluster)
+    assert pick(0.0625, GPU, [2] * 5) == 1  # 4.4, 6.9
+    assert pick(0.0625, GPU, [2] * 64) == 1  # 4.6, 7.5
+    assert pick(0.128, GPU, [3] * 24) == 1  # 5.1, 7.3
+    assert pick(0.128, GPU, [7] * 24) == 4  # 8.3, 7.4
+    assert pick(0.52, GPU, [4] * 5) in (2, 4)
+
+
 def test_every_batch_picks_a_size_that_exists(pick):
     for n in (1, 3, 17, 300):
         for b in (1, 2, 7, 60, 400):
