@@ -779,7 +779,7 @@ struct Engine {
 
   ~Engine() {
     if (args_done) {
-      cudaEventSynchronize(args_done);
+      if (cudaEventSynchronize(args_done) != cudaSuccess) cudaGetLastError();  // (last recorded into a caller's graph)
       cudaEventDestroy(args_done);
     }
     if (stream) cudaStreamSynchronize(stream);
@@ -992,6 +992,14 @@ struct Engine {
     if (prec == HEOM_FP32_MIXED && in.M <= 32 * heom::block_sets(in.N, (int)rsize(), c.block)) return c;
     while (c.team_ctas < 16 && c.team_ctas * 32 < in.M) c.team_ctas <<= 1;
     return c;
+  }
+
+  // Is the caller capturing the stream into a CUDA graph?  The default of a small hierarchy then runs as a cluster
+  // launch: a dataflow launch is made for the tags of one call, and a replay of it can meet words of the run before.
+  bool stream_capturing() const {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &st) != cudaSuccess) cudaGetLastError();  // (the legacy stream during a capture)
+    return st != cudaStreamCaptureStatusNone;
   }
 
   int add_instance(const heom_params& p) {
@@ -1278,6 +1286,7 @@ struct Engine {
       g.sc = std::get<2>(kv.first);
       g.c = cfg[g.N];
       std::vector<int>& ids = kv.second;
+      if (g.c.automatic && stream_capturing()) g.c = cluster_cfg(*inst[ids[0]], 0, 0);
       if (g.N > heom::kMaxSmallN) {
         if (g.c.mode == 2) return fail(HEOM_EINVAL, "launch mode 2 supports at most %d sites", heom::kMaxSmallN);
         g.dyn = heom::large_smem_bytes(g.N, (int)rsize(), g.cplx != 0);
