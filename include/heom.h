@@ -400,7 +400,8 @@ int heom_batch_set_launch(heom_batch* b, int32_t mode, int32_t team_ctas, int32_
                           int32_t node_threads);
 /* Autotuner for a batch: times `trial_steps` steps of every instance for each
  * candidate shape (mode 0 and, in HEOM_FP32_MIXED, mode 2; 256 or 512
- * threads; 1-16 team CTAs; node_threads 1-8), one shape for all site counts;
+ * threads; 1-16 team CTAs; node_threads up to 8, one of those that select the
+ * same kernel), one shape for all site counts;
  * shapes that cannot run every instance are skipped.  Keeps the fastest,
  * restores the state it found and returns that shape's time in *best_ms (may
  * be NULL).  Holds a copy of the batch's state meanwhile. */

@@ -2117,22 +2117,24 @@ int heom_autotune(heom_ctx* ctx, int64_t trial_steps, double* best_us_per_step) 
   CUDA_TRY(cudaMemcpyAsync(sa.p, in.acc.p, in.acc.bytes, cudaMemcpyDeviceToDevice, e.stream));
   std::vector<LaunchCfg> cands;
   const bool large = in.N > heom::kMaxSmallN;
+  const int blockG = in.scaled ? 4 : 2;  // node_threads 1, 2 and 4 are one kernel with one shape: timed once
   for (int G : {1, 2, 4, 8, 16, 32}) {
     if (large && G > 1) break;
+    const bool twin = !large && G <= 4 && G != blockG;  // (in modes 0 and 1)
     for (int block : {128, 256, 512})
       for (int ctas : {1, 2, 4, 8, 16}) {
-        if (block > e.max_block() || (large && block != 256)) continue;
+        if (twin || block > e.max_block() || (large && block != 256)) continue;
         LaunchCfg c;
         c.mode = 0;
         c.team_ctas = ctas;
         c.block = block;
         c.G = G;
-        const int64_t units = ((in.M + 31) / 32) * G;
+        const int64_t units = ((in.M + 31) / 32) * (large ? G : std::max(G, 4));
         if ((int64_t)ctas * block / 32 > 4 * units && ctas > 1) continue;  // mostly idle warps
         cands.push_back(c);
       }
     for (int block : {128, 256, 512}) {
-      if (block > e.max_block() || (large && block != 256)) continue;
+      if (twin || block > e.max_block() || (large && block != 256)) continue;
       LaunchCfg c;
       c.mode = 1;
       c.block = block;
@@ -2142,9 +2144,11 @@ int heom_autotune(heom_ctx* ctx, int64_t trial_steps, double* best_us_per_step) 
     if (!large && G == 1) {
       // the dataflow engine: S nodes per unit row and npt nodes per thread (its unit
       // groups are fixed: one thread per unit); shapes whose CTAs cannot all be resident
-      // are refused by the launch
+      // are refused by the launch.  More nodes per thread than are built run as mode 1
+      // does, and a hierarchy of the one-CTA kernel runs alike in all of them.
       const int U = in.N * (in.N + 1) / 2;
-      for (int npt = 1; npt <= heom::kFlowMaxNpt; ++npt) {
+      const bool one_cta = heom::flow_small_fits(in.N, (int)e.rsize(), in.M);
+      for (int npt = 1; npt <= (one_cta ? 1 : heom::flow_built_npt(in.N)); ++npt) {
         if (!e.flow_kernel_shape(in.complex_h != 0, in.N, npt)) continue;
         const int maxthr = npt == 1 ? heom::kFlowMaxThreads : heom::kFlowMaxThreadsMulti;
         for (int S : {4, 6, 8, 9, 10, 12, 13, 16, 24, 32, 64}) {
@@ -2155,6 +2159,7 @@ int heom_autotune(heom_ctx* ctx, int64_t trial_steps, double* best_us_per_step) 
           c.G = 1;
           c.team_ctas = npt;
           cands.push_back(c);
+          if (one_cta) break;
         }
       }
     }
@@ -2394,6 +2399,11 @@ int heom_batch_autotune(heom_batch* b, int64_t trial_steps, double* best_ms) {
   }
   // candidates: cluster teams on device memory, and on distributed shared memory in mixed precision;
   // one shape for every site count of the batch
+  bool any_small = false, any_scaled = false;
+  for (auto& in : e.inst) {
+    any_small |= in->N <= heom::kMaxSmallN;
+    any_scaled |= in->N <= heom::kMaxSmallN && in->scaled;
+  }
   std::vector<LaunchCfg> cands;
   for (int mode : {0, 2}) {
     if (mode == 2 && e.prec != HEOM_FP32_MIXED) continue;
@@ -2401,6 +2411,8 @@ int heom_batch_autotune(heom_batch* b, int64_t trial_steps, double* best_ms) {
       if (block > e.max_block()) continue;
       for (int ctas : {1, 2, 4, 8, 16})
         for (int G : {1, 2, 4, 8}) {
+          // in mode 0 node_threads 1, 2 and 4 are one kernel, and N > 8 has only one: each timed once
+          if (mode == 0 && G != (any_scaled ? 4 : 2) && (G <= 4 || !any_small)) continue;
           LaunchCfg c;
           c.mode = mode;
           c.team_ctas = ctas;
