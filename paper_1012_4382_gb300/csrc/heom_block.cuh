@@ -50,12 +50,13 @@
 namespace heom {
 
 // Sets (N warps each) of the largest CTA, and the threads the kernels are
-// compiled for.  FP32: three sets at N = 7 (80 registers a thread), two at N = 8
-// (128).  With up to 28 warps (72 registers, 212 bytes of spills read back at N = 7,
-// 172 at N = 8) depth 8 took 15.3 us per step against 13.2, depth 12 37.5 against 35.5,
-// a scan of 256 hierarchies 29.6 ms against 28.6, a serving burst 46.0 ms against 41.8;
-// with 24 the burst 46.0 (three sets at N = 8), with 18 the scan 33.2.  FP64: 144
-// registers at N = 7.
+// compiled for.  FP32: three sets at N = 7 (80 registers a thread, of which 136 bytes
+// spill and 156 are read back), two at N = 8 (128, no spills).  With up to 28 warps (72
+// registers, 212 bytes of spills read back at N = 7, 172 at N = 8) depth 8 took 15.3 us
+// per step against 13.2, depth 12 37.5 against 35.5, a scan of 256 hierarchies 29.6 ms
+// against 28.6, a serving burst 46.0 ms against 41.8; with 24 the burst 46.0 (three sets
+// at N = 8), with 18 the scan 33.2.  FP64: two sets, 128 registers, with 148 bytes of spill
+// stores and 220 of loads at N = 7 (complex H 124 and 136), 388 and 448 at N = 8.
 __host__ __device__ constexpr int block_max_sets(int N, int rsize) {
   const int warps = rsize == 8 ? 16 : 21;
   return warps / N < 1 ? 1 : (warps / N > 14 ? 14 : warps / N);

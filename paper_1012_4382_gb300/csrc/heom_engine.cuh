@@ -63,7 +63,7 @@ struct Inst {
   int32_t dstride;     // distance between the root's diagonal elements in a state array
   const int32_t* up;   // [N][Mpad] index of n + e_j or -1
   const int32_t* dn;   // [N][Mpad] (n_j << 24) | index of n - e_j, or -1
-  void* y;             // packed state (R), see state_elem; N <= 8: ended by a block of zeros
+  void* y;             // packed state (R), see state_elem; ended by a block of zeros
   void* wa;            // stage buffers, same layout
   void* wb;
   // mixed precision: the root node rho in float-float, N*N (hi, lo) float
@@ -295,22 +295,6 @@ __device__ __forceinline__ bool team_barrier(const EngineArgs& A, unsigned& epoc
 // addresses.  Each element is loaded where a unit uses it (the shared view may
 // load the node's whole packed matrix into registers once).
 
-// Loads *a when q holds, else returns 0; predicated, so that gathers of
-// absent neighbours need no branch.
-__device__ __forceinline__ float ld_global_or0(const float* a, bool q) {
-  float v = 0.f;
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q ld.global.f32 %0, [%1];\n\t}"
-               : "+f"(v)
-               : "l"(a), "r"((unsigned)q));
-  return v;
-}
-__device__ __forceinline__ double ld_global_or0(const double* a, bool q) {
-  double v = 0.0;
-  asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.u32 q, %2, 0;\n\t@q ld.global.f64 %0, [%1];\n\t}"
-               : "+d"(v)
-               : "l"(a), "r"((unsigned)q));
-  return v;
-}
 template <typename R>
 struct GlobalArrays {
   const R* __restrict__ win;

@@ -144,7 +144,7 @@ struct ColumnSum<float, NR> {
   __device__ __forceinline__ float2 get(int i) const { return float2{half(re[i / 2], i), half(im[i / 2], i)}; }
 };
 
-// Barrier of `threads` threads; true when `fail` is set on any of them.
+// Barrier of `threads` threads (a set's warps).
 __device__ __forceinline__ void set_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }

@@ -202,7 +202,7 @@ __global__ void bounded_wait_probe_kernel(const unsigned* counter, int* status, 
 }
 
 template <typename R>
-__global__ void set_root_kernel(R* y, int Mpad, float2* y0, const double* rho, int N, double* acc) {
+__global__ void set_root_kernel(R* y, float2* y0, const double* rho, int N, double* acc) {
   const int p = blockIdx.x * blockDim.x + threadIdx.x;
   if (p < N * N) {
     const int a = p / N, b = p - (p / N) * N;
@@ -255,7 +255,7 @@ __global__ void set_roots_kernel(const RootTarget* targets, const double* rho_al
 
 // packed state -> full complex matrices [M][N][N]
 template <typename R>
-__global__ void unpack_state_kernel(const R* y, int Mpad, int64_t M, int N, const float2* y0, double* out) {
+__global__ void unpack_state_kernel(const R* y, int64_t M, int N, const float2* y0, double* out) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int NN = N * N;
   if (idx >= M * NN) return;
@@ -282,7 +282,7 @@ __global__ void unpack_state_kernel(const R* y, int Mpad, int64_t M, int N, cons
 }
 
 template <typename R>
-__global__ void pack_state_kernel(const double* in, R* y, int Mpad, int64_t M, int N, float2* y0) {
+__global__ void pack_state_kernel(const double* in, R* y, int64_t M, int N, float2* y0) {
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int NN = N * N;
   if (idx >= M * NN) return;
@@ -306,7 +306,7 @@ int launch_blocks(int64_t work, int threads) { return (int)((work + threads - 1)
 // Largest element modulus of every node's matrix (packed):
 // out[n] = max_ab |sigma_n,ab|, one thread per node.
 template <typename R>
-__global__ void node_max_kernel(const R* y, int Mpad, int64_t M, int N, double* out) {
+__global__ void node_max_kernel(const R* y, int64_t M, int N, double* out) {
   const int64_t n = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (n >= M) return;
   double mx = 0.0;
@@ -1150,11 +1150,11 @@ struct Engine {
     CUDA_TRY(cudaMemsetAsync(in.y.p, 0, arr, stream));
     const int NN = in.N * in.N;
     if (prec == HEOM_FP64)
-      set_root_kernel<double><<<launch_blocks(NN, 128), 128, 0, stream>>>(in.y.as<double>(), in.Mpad, nullptr, d_rho,
-                                                                         in.N, in.acc.as<double>());
+      set_root_kernel<double><<<launch_blocks(NN, 128), 128, 0, stream>>>(in.y.as<double>(), nullptr, d_rho, in.N,
+                                                                         in.acc.as<double>());
     else
-      set_root_kernel<float><<<launch_blocks(NN, 128), 128, 0, stream>>>(in.y.as<float>(), in.Mpad, root_ptr(in, 0),
-                                                                        d_rho, in.N, in.acc.as<double>());
+      set_root_kernel<float><<<launch_blocks(NN, 128), 128, 0, stream>>>(in.y.as<float>(), root_ptr(in, 0), d_rho, in.N,
+                                                                        in.acc.as<double>());
     CUDA_TRY(cudaGetLastError());
     return HEOM_OK;
   }
@@ -1764,10 +1764,10 @@ struct Engine {
     TRY(tmp.alloc(bytes, hooks));
     const int64_t work = M * in.N * in.N;
     if (prec == HEOM_FP64)
-      unpack_state_kernel<double><<<launch_blocks(work, 256), 256, 0, stream>>>(in.y.as<double>(), in.Mpad, M, in.N,
+      unpack_state_kernel<double><<<launch_blocks(work, 256), 256, 0, stream>>>(in.y.as<double>(), M, in.N,
                                                                                nullptr, tmp.as<double>());
     else
-      unpack_state_kernel<float><<<launch_blocks(work, 256), 256, 0, stream>>>(in.y.as<float>(), in.Mpad, M, in.N,
+      unpack_state_kernel<float><<<launch_blocks(work, 256), 256, 0, stream>>>(in.y.as<float>(), M, in.N,
                                                                               root_ptr(in, 0), tmp.as<double>());
     CUDA_TRY(cudaGetLastError());
     CUDA_TRY(cudaStreamSynchronize(stream));
@@ -1790,10 +1790,10 @@ struct Engine {
     const int64_t work = in.M * in.N * in.N;
     if (prec == HEOM_FP64)
       pack_state_kernel<double><<<launch_blocks(work, 256), 256, 0, stream>>>(tmp.as<double>(), in.y.as<double>(),
-                                                                             in.Mpad, in.M, in.N, nullptr);
+                                                                             in.M, in.N, nullptr);
     else
       pack_state_kernel<float><<<launch_blocks(work, 256), 256, 0, stream>>>(tmp.as<double>(), in.y.as<float>(),
-                                                                            in.Mpad, in.M, in.N, root_ptr(in, 0));
+                                                                            in.M, in.N, root_ptr(in, 0));
     CUDA_TRY(cudaGetLastError());
     double acc[kAccDoubles] = {extra ? extra[0] : 0.0, extra ? extra[1] : 0.0};
     CUDA_TRY(cudaMemcpyAsync(in.acc.p, acc, sizeof(acc), cudaMemcpyHostToDevice, stream));
@@ -1927,10 +1927,10 @@ int heom_node_magnitudes(heom_ctx* ctx, double* node_max) {
   const size_t need = sizeof(double) * (size_t)in.M;
   if (e.d_out.bytes < need) TRY(e.d_out.alloc(need, e.hooks));
   if (e.prec == HEOM_FP64)
-    node_max_kernel<double><<<launch_blocks(in.M, 256), 256, 0, e.stream>>>(in.y.as<double>(), in.Mpad, in.M, in.N,
+    node_max_kernel<double><<<launch_blocks(in.M, 256), 256, 0, e.stream>>>(in.y.as<double>(), in.M, in.N,
                                                                           e.d_out.as<double>());
   else
-    node_max_kernel<float><<<launch_blocks(in.M, 256), 256, 0, e.stream>>>(in.y.as<float>(), in.Mpad, in.M, in.N,
+    node_max_kernel<float><<<launch_blocks(in.M, 256), 256, 0, e.stream>>>(in.y.as<float>(), in.M, in.N,
                                                                          e.d_out.as<double>());
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaStreamSynchronize(e.stream));
@@ -2265,10 +2265,10 @@ int heom_batch_node_magnitudes(heom_batch* b, int32_t i, double* node_max) {
   const size_t need = sizeof(double) * (size_t)in.M;
   if (e.d_out.bytes < need) TRY(e.d_out.alloc(need, e.hooks));
   if (e.prec == HEOM_FP64)
-    node_max_kernel<double><<<launch_blocks(in.M, 256), 256, 0, e.stream>>>(in.y.as<double>(), in.Mpad, in.M, in.N,
+    node_max_kernel<double><<<launch_blocks(in.M, 256), 256, 0, e.stream>>>(in.y.as<double>(), in.M, in.N,
                                                                           e.d_out.as<double>());
   else
-    node_max_kernel<float><<<launch_blocks(in.M, 256), 256, 0, e.stream>>>(in.y.as<float>(), in.Mpad, in.M, in.N,
+    node_max_kernel<float><<<launch_blocks(in.M, 256), 256, 0, e.stream>>>(in.y.as<float>(), in.M, in.N,
                                                                          e.d_out.as<double>());
   CUDA_TRY(cudaGetLastError());
   CUDA_TRY(cudaStreamSynchronize(e.stream));
@@ -2694,10 +2694,10 @@ extern "C" int heom_propagate_static(const heom_params* params, const double* d_
   CUDA_TRY(cudaMemcpyAsync(base + o_team, team, sizeof(team), cudaMemcpyHostToDevice, stream));
   const int NN = N * N;
   if (fp64)
-    set_root_kernel<double><<<launch_blocks(NN, 128), 128, 0, stream>>>(static_cast<double*>(d.y), Mpad, nullptr,
+    set_root_kernel<double><<<launch_blocks(NN, 128), 128, 0, stream>>>(static_cast<double*>(d.y), nullptr,
                                                                        d_rho0, N, d.acc);
   else
-    set_root_kernel<float><<<launch_blocks(NN, 128), 128, 0, stream>>>(static_cast<float*>(d.y), Mpad,
+    set_root_kernel<float><<<launch_blocks(NN, 128), 128, 0, stream>>>(static_cast<float*>(d.y),
                                                                       static_cast<float2*>(d.y0), d_rho0, N, d.acc);
   CUDA_TRY(cudaGetLastError());
 
@@ -2715,10 +2715,10 @@ extern "C" int heom_propagate_static(const heom_params* params, const double* d_
   CUDA_TRY(cudaLaunchKernelExC(&lc, k, args));
   if (d_rho_out) {
     if (fp64)
-      unpack_state_kernel<double><<<launch_blocks(NN, 128), 128, 0, stream>>>(static_cast<double*>(d.y), Mpad, 1, N,
+      unpack_state_kernel<double><<<launch_blocks(NN, 128), 128, 0, stream>>>(static_cast<double*>(d.y), 1, N,
                                                                              nullptr, d_rho_out);
     else
-      unpack_state_kernel<float><<<launch_blocks(NN, 128), 128, 0, stream>>>(static_cast<float*>(d.y), Mpad, 1, N,
+      unpack_state_kernel<float><<<launch_blocks(NN, 128), 128, 0, stream>>>(static_cast<float*>(d.y), 1, N,
                                                                             static_cast<const float2*>(d.y0),
                                                                             d_rho_out);
     CUDA_TRY(cudaGetLastError());
@@ -2900,9 +2900,8 @@ struct heom_server {
     while (c < 16 && (int64_t)c * 256 < M) c <<= 1;
     return c;
   }
-  // Launch shape of a request: the throughput engine.  (Smaller teams -- 2 CTAs, or the fewest whose shared
-  // memory holds the hierarchy -- were measured slower on the serving trace:
-  // the largest requests' service time then sets the makespan.)
+  // Launch shape of a request: the throughput engine.  (Other sizes -- 96, 128 or 512 nodes per CTA -- move a burst by
+  // less than 1 %: the largest request on the largest team sets its time.)
   static LaunchCfg launch_for(int prec, int N, int64_t M, bool scaled) {
     LaunchCfg c;
     c.mode = 0;
