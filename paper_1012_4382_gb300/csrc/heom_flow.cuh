@@ -334,9 +334,12 @@ __global__ void __launch_bounds__(NPT == 1 ? kFlowMaxThreads : kFlowMaxThreadsMu
   // anyway: with the blocked index computed from p and n the compiler kept addresses of both alive over the loop, in
   // registers that the FP64 and complex kernels do not have (us per step, FP64, complex H: 8 sites depth 4 19.3 against
   // 14.9, seven sites depth 6 25.9 against 25.2; mixed: seven sites depth 6 complex 5.9 against 5.2, 5 sites depth 12 10.4
-  // against 8.2).
-  auto blocked = [&I](int o) {
-    const int p = o / I.Mpad, n = o - p * I.Mpad;
+  // against 8.2).  Three sites with real H in mixed precision do have them: depth 9 4.6 us a step that way, 4.85 this way.
+  auto blocked = [&I](int o, int p, int n) {
+    if constexpr (!(MIXED && !CPLX && N == 3)) {
+      p = o / I.Mpad;
+      n = o - p * I.Mpad;
+    }
     return node_col<N>(n) + p * 32;
   };
   const R* gy = static_cast<const R*>(I.y);
@@ -345,8 +348,8 @@ __global__ void __launch_bounds__(NPT == 1 ? kFlowMaxThreads : kFlowMaxThreadsMu
     y_r[k] = y_i[k] = R(0);
     if (!valid[k]) continue;
     const int oab = pab * Mp + nd[k], oba = pba * Mp + nd[k];
-    y_r[k] = gy[blocked(oab)];
-    y_i[k] = pair ? gy[blocked(oba)] : R(0);
+    y_r[k] = gy[blocked(oab, pab, nd[k])];
+    y_i[k] = pair ? gy[blocked(oba, pba, nd[k])] : R(0);
     R* own = sb + (k * S + l) * NN;
     own[pab] = y_r[k];
     if (pair) own[pba] = y_i[k];
@@ -592,8 +595,8 @@ __global__ void __launch_bounds__(NPT == 1 ? kFlowMaxThreads : kFlowMaxThreadsMu
   for (int k = 0; k < NPT; ++k) {
     if (!valid[k]) continue;
     const int oab = pab * Mp + nd[k], oba = pba * Mp + nd[k];
-    gyw[blocked(oab)] = y_r[k];
-    if (pair) gyw[blocked(oba)] = y_i[k];
+    gyw[blocked(oab, pab, nd[k])] = y_r[k];
+    if (pair) gyw[blocked(oba, pba, nd[k])] = y_i[k];
   }
   if constexpr (MIXED) {
     if (root) {
@@ -619,8 +622,10 @@ __global__ void __launch_bounds__(NPT == 1 ? kFlowMaxThreads : kFlowMaxThreadsMu
 // of a pair are separate threads, terms that are zero in a whole warp are
 // skipped, and the output rows (sums and conversions in double) are left to one
 // more warp.  us per step with a row every step, two sites, depth 4, FP64: 10.2 as
-// a cluster launch of the load views, 8.4 of the throughput engine, 3.4 here;
-// seven sites, depth 3: mixed 24.5 -> 5.3, FP64 52 -> 10.3.
+// a cluster launch of the load views, 8.4 of the throughput engine, 3.4 here.  Without
+// rows, load views before and here: two sites depth 19 (840 reals) mixed 6.6, 2.6; four
+// sites depth 3 (560) mixed 8.6, 2.5; seven sites depth 1 (392) mixed 20.2, 3.2; two sites
+// depth 9 (220) FP64 9.0, 4.5.
 template <int N, typename R, bool CPLX>
 __host__ __device__ constexpr int flow_small_terms() {
   return (flow_nre(N, CPLX) > flow_nim(N, CPLX) ? flow_nre(N, CPLX) : flow_nim(N, CPLX)) + 6;
