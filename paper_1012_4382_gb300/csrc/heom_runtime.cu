@@ -872,6 +872,10 @@ struct Engine {
     for (int i = 0; i < 5; ++i) {
       resident[i] = sms / heom::kTeamSizes[i];
       if (!batch) continue;  // (a server gives its launches a shape of their own)
+      if (i > 0 && heom::kTeamSizes[i - 1] * (int64_t)32 >= Mmax) {
+        resident[i] = 0;  // no more blocks to spread than the size before takes at once
+        continue;
+      }
       LaunchCfg c;
       c.mode = 0;
       c.team_ctas = heom::kTeamSizes[i];
