@@ -69,15 +69,16 @@ __host__ __device__ constexpr int large_smem_bytes(int N, int rsize, bool cplx) 
          large_sets(N, rsize) * (large_stage_bytes(N, rsize) + large_exch_bytes(N, rsize));
 }
 
-// Parts in which a team of `team` CTAs with `sets` sets each computes its last `rest` < sets * team blocks: the fewest
-// that make the CTA with the most parts' share of a block smallest (a CTA's sets share its FP64 pipe, so a second busy
-// set gains nothing by itself: 16 sites depth 4, 152 blocks on 152 CTAs, in halves 407 us a step against 370), a smaller
-// share by less than 5 % not counted; at least three columns a part.
+// Parts in which a team of `team` CTAs with `sets` sets each computes its last `rest` < sets * team blocks, at least three
+// columns a part: those that make the largest share of a block on one CTA smallest.  A CTA's sets share its FP64 pipe, so
+// sharing must save a CTA 5 % to be worth its extra reads (16 sites depth 4, 152 blocks on 152 CTAs, in halves 407 us a
+// step against 370), but of two counts with the same share the larger keeps more sets busy (12 sites depth 4, 57 blocks:
+// a half per CTA 122 us, two quarters 107).
 __host__ __device__ constexpr int large_parts(int N, int sets, int team, int rest) {
   int best = 1, most = rest > 0 ? (rest + team - 1) / team : 1;  // parts, and those of the fullest CTA
   for (int p = 2; p <= N / 3 && p * rest <= sets * team; ++p) {
     const int m = (rest * p + team - 1) / team;
-    if (20 * m * best < 19 * most * p) {
+    if (best == 1 ? 20 * m < 19 * most * p : m * best <= most * p) {
       best = p;
       most = m;
     }
